@@ -32,6 +32,7 @@ struct KernelJob {
   uint32_t oob_slot;  // index of the job's out-of-bounds records (IGS_MAX_ACCESSORS of them)
   uint32_t lo[3], hi[3];  // chunk box (kernel index space)
   uint32_t params[4];
+  uint32_t lanes;  // N-body step: lanes per body (igs_nbody_lanes)
   uint64_t item_begin;
   KAcc acc[IGS_MAX_ACCESSORS];
 };
@@ -42,11 +43,11 @@ struct KernelJob {
 enum FlowKind : uint32_t { FK_NONE = 0, FK_COPY = 1, FK_STENCIL = 2, FK_WORKLOAD = 3 };
 
 // Tile sizes: a stencil tile is kFlowStencilRows rows of a strip of
-// kFlowThreads groups of four columns; workload items; N-body bodies.
+// kFlowThreads groups of four columns; workload items. An N-body tile is
+// kFlowThreads / lanes bodies.
 constexpr uint32_t kFlowThreads = 256;
 constexpr uint32_t kFlowStencilRows = 16;
 constexpr uint32_t kFlowItems = 1024;
-constexpr uint32_t kFlowBodies = kFlowThreads;
 
 struct FlowNode {
   uint32_t kind, first, count;  // jobs [first, first + count) of the copy or kernel job array
@@ -78,6 +79,11 @@ int igs_launch_flow(igs::FlowCtl* ctl, igs::FlowNode* nodes, uint32_t n_nodes, c
 // Loads the execution kernels' code now (once per process).
 void igs_exec_preload();
 int igs_launch_workload(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint64_t n_items, void* stream);
+// N-body step jobs of up to max_bodies bodies each, all with the given lanes
+// per body; n_jobs <= 65535.
+int igs_launch_nbody(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint32_t max_bodies, uint32_t lanes, void* stream);
+// Lanes per body for N-body jobs that run together over `bodies` bodies.
+uint32_t igs_nbody_lanes(uint64_t bodies);
 // 5-point stencil jobs (Jacobi / wave), pre-validated by the host; n_jobs <= 65535.
 int igs_launch_stencil(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint64_t max_items, void* stream);
 // One level's stencil jobs and box-copy units in one launch (they are

@@ -978,9 +978,9 @@ namespace {
 // launch; frees follow the launches of their level.
 struct LevelWork {
   std::vector<CopyJob> copies;
-  std::vector<KernelJob> kernels, stencils;
+  std::vector<KernelJob> kernels, stencils, nbodies;
   std::vector<void*> frees;
-  uint64_t copy_units = 0, kernel_items = 0, stencil_max = 0;
+  uint64_t copy_units = 0, kernel_items = 0, stencil_max = 0, bodies = 0, bodies_max = 0;
 };
 
 // The dataflow graph of one execute call: a node per walked instruction, its
@@ -1093,6 +1093,12 @@ void add_kernel(Pending& p, uint32_t L, KernelJob J, uint64_t items, bool stenci
     w.stencil_max = std::max(w.stencil_max, items);
     return;
   }
+  if (J.kernel == K_NBODY_STEP) {
+    w.nbodies.push_back(J);
+    w.bodies += J.hi[0] - J.lo[0];
+    w.bodies_max = std::max<uint64_t>(w.bodies_max, J.hi[0] - J.lo[0]);
+    return;
+  }
   J.item_begin = w.kernel_items;
   w.kernel_items += items;
   w.kernels.push_back(J);
@@ -1198,15 +1204,15 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
   size_t ncj = 0, nkj = 0;
   for (const LevelWork& w : p.levels) {
     ncj += w.copies.size();
-    nkj += w.kernels.size() + w.stencils.size();
+    nkj += w.kernels.size() + w.stencils.size() + w.nbodies.size();
   }
-  std::vector<size_t> co(p.levels.size()), ko(p.levels.size()), so(p.levels.size());
+  std::vector<size_t> co(p.levels.size()), ko(p.levels.size()), so(p.levels.size()), bo(p.levels.size());
   int r;
   if ((r = grow_pinned(c, c->h_cjobs[k], c->hcap_cjobs[k], std::max<size_t>(ncj, 1)))) return r;
   if ((r = grow_pinned(c, c->h_kjobs[k], c->hcap_kjobs[k], std::max<size_t>(nkj, 1)))) return r;
   size_t nc = 0, nk = 0;
   for (size_t L = 0; L < p.levels.size(); ++L) {
-    const LevelWork& w = p.levels[L];
+    LevelWork& w = p.levels[L];
     co[L] = nc;
     std::copy(w.copies.begin(), w.copies.end(), c->h_cjobs[k] + nc);
     nc += w.copies.size();
@@ -1216,6 +1222,11 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
     so[L] = nk;
     std::copy(w.stencils.begin(), w.stencils.end(), c->h_kjobs[k] + nk);
     nk += w.stencils.size();
+    bo[L] = nk;
+    const uint32_t lanes = w.nbodies.empty() ? 1u : igs_nbody_lanes(w.bodies);
+    for (KernelJob& J : w.nbodies) J.lanes = lanes;
+    std::copy(w.nbodies.begin(), w.nbodies.end(), c->h_kjobs[k] + nk);
+    nk += w.nbodies.size();
   }
   if ((r = oob_prepare(c, c->h_kjobs[k], nk, p.oob_first, s))) return r;
   if (nc) {
@@ -1260,6 +1271,14 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
       const size_t ev = c->timing ? ev_begin(c, s) : 0;
       if (igs_launch_workload(c->d_kjobs[k] + ko[L], (uint32_t)w.kernels.size(), w.kernel_items, s))
         return fail_ctx(c, IGS_ERR_CUDA, "workload launch");
+      if (c->timing) ev_end(c, 2, ev, s);
+      c->n_launch[2]++;
+    }
+    for (size_t first = 0; first < w.nbodies.size(); first += 65535) {
+      const uint32_t n = (uint32_t)std::min<size_t>(65535, w.nbodies.size() - first);
+      const size_t ev = c->timing ? ev_begin(c, s) : 0;
+      if (igs_launch_nbody(c->d_kjobs[k] + bo[L] + first, n, (uint32_t)w.bodies_max, w.nbodies[0].lanes, s))
+        return fail_ctx(c, IGS_ERR_CUDA, "N-body launch");
       if (c->timing) ev_end(c, 2, ev, s);
       c->n_launch[2]++;
     }
@@ -1352,10 +1371,16 @@ int run_flow(igs_ctx* c, FlowBuild& g, cudaStream_t s, bool wait) {
       const uint32_t strips = ((J.hi[1] - J.lo[1] + 3) / 4 + kFlowThreads - 1) / kFlowThreads;
       f.tiles = strips * ((J.hi[0] - J.lo[0] + kFlowStencilRows - 1) / kFlowStencilRows);
     } else if (f.kind == FK_WORKLOAD) {
-      const KernelJob& J = g.kernels[f.first];
+      KernelJob& J = g.kernels[f.first];
       const uint64_t items = (uint64_t)(J.hi[0] - J.lo[0]) * (J.hi[1] - J.lo[1]) * (J.hi[2] - J.lo[2]);
-      f.tiles = J.kernel == K_NBODY_STEP ? (J.hi[0] - J.lo[0] + kFlowBodies - 1) / kFlowBodies
-                                         : (uint32_t)((items + kFlowItems - 1) / kFlowItems);
+      if (J.kernel == K_NBODY_STEP) {
+        // the kernels of one step run together: about all the bodies
+        J.lanes = igs_nbody_lanes(J.acc[0].ext[0]);
+        const uint32_t per = kFlowThreads / J.lanes;
+        f.tiles = (J.hi[0] - J.lo[0] + per - 1) / per;
+      } else {
+        f.tiles = (uint32_t)((items + kFlowItems - 1) / kFlowItems);
+      }
     } else if (f.kind == FK_NONE) {
       f.tiles = 1;
     }
