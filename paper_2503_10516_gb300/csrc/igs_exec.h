@@ -32,7 +32,7 @@ struct KernelJob {
   uint32_t oob_slot;  // index of the job's out-of-bounds records (IGS_MAX_ACCESSORS of them)
   uint32_t lo[3], hi[3];  // chunk box (kernel index space)
   uint32_t params[4];
-  uint32_t lanes;  // N-body step: lanes per body (igs_nbody_lanes)
+  uint32_t lanes;  // N-body step: lanes per body (igs_nbody_lanes); stencils: rows of a tile (igs_stencil_rows)
   uint64_t item_begin;
   KAcc acc[IGS_MAX_ACCESSORS];
 };
@@ -42,10 +42,11 @@ struct KernelJob {
 // tiles that any block may run once every predecessor node has finished.
 enum FlowKind : uint32_t { FK_NONE = 0, FK_COPY = 1, FK_STENCIL = 2, FK_WORKLOAD = 3 };
 
-// Tile sizes: a stencil tile is kFlowStencilRows rows of a strip of
-// kFlowThreads groups of four columns; workload items. An N-body tile is
-// kFlowThreads / lanes bodies.
+// Tile sizes: a stencil tile is kStencilWarps strips of 128 columns, `lanes`
+// rows each (kFlowStencilRows in a dataflow launch); workload items. An N-body
+// tile is kFlowThreads / lanes bodies.
 constexpr uint32_t kFlowThreads = 256;
+constexpr uint32_t kStencilWarps = 8;  // warps of a stencil block
 constexpr uint32_t kFlowStencilRows = 16;
 constexpr uint32_t kFlowItems = 1024;
 
@@ -84,12 +85,17 @@ int igs_launch_workload(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint64_
 int igs_launch_nbody(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint32_t max_bodies, uint32_t lanes, void* stream);
 // Lanes per body for N-body jobs that run together over `bodies` bodies.
 uint32_t igs_nbody_lanes(uint64_t bodies);
-// 5-point stencil jobs (Jacobi / wave), pre-validated by the host; n_jobs <= 65535.
-int igs_launch_stencil(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint64_t max_items, void* stream);
+// Block tiles of a stencil job at `rows` rows a tile, and the rows of a tile
+// for jobs that run in one launch.
+uint32_t igs_stencil_tiles(const igs::KernelJob& J, uint32_t rows);
+uint32_t igs_stencil_rows(const igs::KernelJob* jobs, size_t n);
+// 5-point stencil jobs (Jacobi / wave), pre-validated by the host, of at most
+// max_tiles block tiles each; n_jobs <= 65535.
+int igs_launch_stencil(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint32_t max_tiles, void* stream);
 // One level's stencil jobs and box-copy units in one launch (they are
 // independent by construction of the levels). -1 when the grid would exceed
 // 65535 rows (the caller then launches them separately).
-int igs_launch_level(const igs::KernelJob* sjobs_dev, uint32_t n_sjobs, uint64_t max_items,
+int igs_launch_level(const igs::KernelJob* sjobs_dev, uint32_t n_sjobs, uint32_t max_tiles,
                      const igs::CopyJob* cjobs_dev, uint32_t n_cjobs, uint64_t n_units, void* stream);
 // Execution error flags (0 = none; bit 0: a workload kernel met an index
 // outside its allocation, bit 1: a dataflow launch gave up waiting);

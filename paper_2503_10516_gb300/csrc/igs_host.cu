@@ -980,7 +980,8 @@ struct LevelWork {
   std::vector<CopyJob> copies;
   std::vector<KernelJob> kernels, stencils, nbodies;
   std::vector<void*> frees;
-  uint64_t copy_units = 0, kernel_items = 0, stencil_max = 0, bodies = 0, bodies_max = 0;
+  uint64_t copy_units = 0, kernel_items = 0, bodies = 0, bodies_max = 0;
+  uint32_t stencil_tiles = 0;  // block tiles of the largest stencil job
 };
 
 // The dataflow graph of one execute call: a node per walked instruction, its
@@ -1090,7 +1091,6 @@ void add_kernel(Pending& p, uint32_t L, KernelJob J, uint64_t items, bool stenci
   LevelWork& w = p.at(L);
   if (stencil) {
     w.stencils.push_back(J);
-    w.stencil_max = std::max(w.stencil_max, items);
     return;
   }
   if (J.kernel == K_NBODY_STEP) {
@@ -1220,6 +1220,13 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
     std::copy(w.kernels.begin(), w.kernels.end(), c->h_kjobs[k] + nk);
     nk += w.kernels.size();
     so[L] = nk;
+    if (!w.stencils.empty()) {
+      const uint32_t rows = igs_stencil_rows(w.stencils.data(), w.stencils.size());
+      for (KernelJob& J : w.stencils) {
+        J.lanes = rows;
+        w.stencil_tiles = std::max(w.stencil_tiles, igs_stencil_tiles(J, rows));
+      }
+    }
     std::copy(w.stencils.begin(), w.stencils.end(), c->h_kjobs[k] + nk);
     nk += w.stencils.size();
     bo[L] = nk;
@@ -1244,7 +1251,7 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
     // workload time and its copy bytes are not in copy_bytes
     if (!w.copies.empty() && !w.stencils.empty() && w.stencils.size() + 2048 <= 65535) {
       const size_t ev = c->timing ? ev_begin(c, s) : 0;
-      if (igs_launch_level(c->d_kjobs[k] + so[L], (uint32_t)w.stencils.size(), w.stencil_max, c->d_cjobs[k] + co[L],
+      if (igs_launch_level(c->d_kjobs[k] + so[L], (uint32_t)w.stencils.size(), w.stencil_tiles, c->d_cjobs[k] + co[L],
                            (uint32_t)w.copies.size(), w.copy_units, s))
         return fail_ctx(c, IGS_ERR_CUDA, "level launch");
       if (c->timing) ev_end(c, 2, ev, s);
@@ -1261,7 +1268,7 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
       for (size_t first = 0; first < w.stencils.size(); first += 65535) {
         const uint32_t n = (uint32_t)std::min<size_t>(65535, w.stencils.size() - first);
         const size_t ev = c->timing ? ev_begin(c, s) : 0;
-        if (igs_launch_stencil(c->d_kjobs[k] + so[L] + first, n, w.stencil_max, s))
+        if (igs_launch_stencil(c->d_kjobs[k] + so[L] + first, n, w.stencil_tiles, s))
           return fail_ctx(c, IGS_ERR_CUDA, "stencil launch");
         if (c->timing) ev_end(c, 2, ev, s);
         c->n_launch[2]++;
@@ -1367,9 +1374,9 @@ int run_flow(igs_ctx* c, FlowBuild& g, cudaStream_t s, bool wait) {
     f.succ_cnt = off[i + 1] - off[i];
     if (f.kind == FK_COPY && f.count == 0) f.kind = FK_NONE;
     if (f.kind == FK_STENCIL) {
-      const KernelJob& J = g.kernels[f.first];
-      const uint32_t strips = ((J.hi[1] - J.lo[1] + 3) / 4 + kFlowThreads - 1) / kFlowThreads;
-      f.tiles = strips * ((J.hi[0] - J.lo[0] + kFlowStencilRows - 1) / kFlowStencilRows);
+      KernelJob& J = g.kernels[f.first];
+      J.lanes = kFlowStencilRows;
+      f.tiles = igs_stencil_tiles(J, kFlowStencilRows);
     } else if (f.kind == FK_WORKLOAD) {
       KernelJob& J = g.kernels[f.first];
       const uint64_t items = (uint64_t)(J.hi[0] - J.lo[0]) * (J.hi[1] - J.lo[1]) * (J.hi[2] - J.lo[2]);

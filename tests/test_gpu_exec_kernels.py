@@ -58,3 +58,48 @@ def test_nbody_step_tiles(n, far, executor):
     c.close()
     for i in sorted({0, n // 3, n // 2, n - 1, min(n - 1, 63), min(n - 1, 64)} | {(7 + 61 * k) % n for k in range(4)}):
         assert np.array_equal(got[i], _nbody_velocity(P, V, i), equal_nan=True), (n, i)
+
+
+def _stencil_reference(prog):
+    """The stencil program's buffers, step by step in float32."""
+    bufs = [None if b.init is None else b.init.astype(np.float32).copy() for b in prog.buffers]
+    for t in prog.tasks:
+        ids = [a.buffer for a in t.accessors]
+        u = bufs[ids[-2]]
+        out = u.copy()
+        if min(u.shape) > 2:
+            n, s, w, e, c = u[:-2, 1:-1], u[2:, 1:-1], u[1:-1, :-2], u[1:-1, 2:], u[1:-1, 1:-1]
+            t5 = (n + s) + (w + e)
+            if len(ids) == 2:
+                out[1:-1, 1:-1] = t5 * np.float32(0.25)
+            else:
+                t2 = np.float32(2.0) * c - bufs[ids[0]][1:-1, 1:-1]
+                out[1:-1, 1:-1] = t2 + np.float32(0.25) * (t5 - np.float32(4.0) * c)
+        bufs[ids[-1]] = out
+    return bufs
+
+
+@pytest.mark.parametrize("executor", [0, 1])
+@pytest.mark.parametrize("kind", ["jacobi", "wave"])
+@pytest.mark.parametrize("shape", [(1, 1), (3, 2), (5, 127), (4, 128), (40, 129), (33, 131), (65, 256), (70, 260),
+                                   (130, 516), (37, 1028), (19, 1031), (513, 2052)], ids=str)
+@pytest.mark.parametrize("chunks", [1, 5, (2 << 16) | 3])
+def test_stencil_strips(shape, chunks, kind, executor):
+    """Stencil strips at ragged and vector widths, heights around the tiles'
+    rows, splits along rows and along both dimensions (whose allocations start
+    at any column), three steps."""
+    make = W.jacobi_program if kind == "jacobi" else W.wave_program
+    prog = make(n=4, steps=3, nodes=1, devices=2, chunks=chunks, lookahead=0)
+    rng = np.random.default_rng(shape[0] * 4096 + shape[1])
+    for b in prog.buffers:
+        b.extent = (*shape, 1)
+        if b.init is not None:
+            b.init = rng.random(shape, dtype=np.float32)
+    for t in prog.tasks:
+        t.range = (*shape, 1)
+    want = _stencil_reference(prog)
+    c = _run(prog, executor)
+    for i, w in enumerate(want):
+        got = c.read_buffer(i, (0, 0, 0), (*shape, 1), 4).view(np.float32).reshape(shape)
+        assert np.array_equal(got, w), (shape, i)
+    c.close()
