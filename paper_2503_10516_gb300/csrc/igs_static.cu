@@ -18,18 +18,27 @@
 
 namespace {
 
-// The scratch every call shares: 32 MiB per device that loads the library,
-// held until the process exits. Calls that overlap on the GPU race on it.
+// The scratch every call shares: 32 MiB (and the words read back) per device
+// that loads the library, held until the process exits. Calls that overlap on the GPU race on it.
 constexpr size_t kStaticBytes = 32u << 20;
-__device__ __align__(256) uint8_t g_static_scratch[kStaticBytes];
+__device__ __align__(256) uint8_t g_static_scratch[kStaticBytes + 256];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 uint8_t* g_base[kMaxDevices] = {};
+uint8_t* g_helpers[kMaxDevices] = {};
 
 // Per-node capacities of this variant (modest, fixed).
 constexpr uint32_t kBuffers = 16, kHeap = 1u << 15, kSlots = 128, kQr = 2048, kScratch = 1024;
 constexpr uint32_t kAlloc = 4096, kQueue = 4096, kRej = 256;
+
+// Scratch of the warps that share a node's lowering (helper warps and the
+// front warp of igs_lower.cu), for programs of at most kHelpedNodes nodes: 42
+// MiB. Programs of more nodes already fill as many SMs with one warp each.
+constexpr uint32_t kHelpedNodes = 8;
+constexpr size_t kHelperBytes =
+    (size_t)igs::kScratchSets * igs::kHelperTables * igs::F_COUNT * kScratch * sizeof(uint32_t);
+__device__ __align__(256) uint8_t g_static_helpers[kHelpedNodes * kHelperBytes];
 
 size_t tbytes(uint32_t cap) { return (size_t)igs::F_COUNT * cap * sizeof(uint32_t); }
 
@@ -57,6 +66,40 @@ Layout layout(uint32_t cap_instr) {
   L.o_scr = take(tbytes(kScratch) * 14);
   L.per_node = p;
   return L;
+}
+
+// What a node's state starts with (the arrays keep the previous call's
+// contents): block n resets node n.
+__global__ void static_init(const igs::NodeDev* nodes) {
+  using namespace igs;
+  const NodeDev nd = nodes[blockIdx.x];
+  const uint32_t desc = kDesc * (2 * kBuffers + 2 * kSlots);
+  for (uint32_t i = threadIdx.x; i < desc; i += blockDim.x) nd.own_d[i] = 0;
+  for (uint32_t i = threadIdx.x; i < kSlots; i += blockDim.x) nd.free_slots[i] = kSlots - 1 - i;  // pops 0, 1, 2, ...
+  if (threadIdx.x == 0) {
+    nd.has_succ[0] = 0;
+    nd.instrs[0] = igs_instruction{0, IGS_EPOCH, NONE, NONE, NONE, NONE, NONE, 0, 0, 0, 0};
+  }
+}
+
+// Counts and status of every node into the caller's words, and what the host
+// reads back: {status, rejected tasks} per node.
+struct CountPtrs {
+  uint32_t* p[32];
+};
+__global__ void static_counts(const igs::NodeDev* nodes, uint32_t n, CountPtrs counts, uint32_t* result) {
+  const uint32_t i = threadIdx.x;
+  if (i >= n) return;
+  const igs::NodeDev& nd = nodes[i];
+  uint32_t* c = counts.p[i];
+  c[0] = nd.n_instr;
+  c[1] = nd.n_edge;
+  c[2] = nd.n_box;
+  c[3] = nd.n_bind;
+  c[4] = nd.n_diag;
+  c[5] = nd.status;
+  result[2 * i] = nd.status;
+  result[2 * i + 1] = nd.n_rej;
 }
 
 }  // namespace
@@ -88,7 +131,7 @@ extern "C" int igs_lower_static(const igs_config* cfg, const igs_static_buffer* 
   cudaStream_t stream = (cudaStream_t)stream_ptr;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return IGS_ERR_CUDA;
-  uint8_t* base = nullptr;
+  uint8_t *base = nullptr, *helpers = nullptr;
   {
     // set-up, once per device, with that device current: the array's device
     // address (the symbol itself is only a host-side stand-in)
@@ -96,9 +139,13 @@ extern "C" int igs_lower_static(const igs_config* cfg, const igs_static_buffer* 
     if (!g_base[dev]) {
       void* p = nullptr;
       if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return IGS_ERR_CUDA;
+      void* h = nullptr;
+      if (cudaGetSymbolAddress(&h, g_static_helpers) != cudaSuccess || !h) return IGS_ERR_CUDA;
       g_base[dev] = static_cast<uint8_t*>(p);
+      g_helpers[dev] = static_cast<uint8_t*>(h);
     }
     base = g_base[dev];
+    helpers = g_helpers[dev];
   }
   uint32_t cap_instr = 0xFFFFFFFFu;
   for (uint32_t n = 0; n < N; ++n) {
@@ -178,14 +225,16 @@ extern "C" int igs_lower_static(const igs_config* cfg, const igs_static_buffer* 
   const size_t o_bufs = take(sizeof(BufDesc) * (num_buffers + 1));
   const size_t o_state = take(L.per_node * N);
   if (off > kStaticBytes) return IGS_ERR_CAPACITY;  // program or instruction capacity too large for the array
-  std::vector<NodeDev> nodes(N);
-  std::vector<Unit> units(N);
-  std::vector<uint32_t> slots(kSlots);
-  for (uint32_t i = 0; i < kSlots; ++i) slots[i] = kSlots - 1 - i;
+  const size_t o_result = kStaticBytes;  // behind the scratch
+  // the inputs, laid out as in the array: one copy takes them there
+  std::vector<uint8_t> stage(o_state);
+  NodeDev* nodes = reinterpret_cast<NodeDev*>(stage.data() + o_nodes);
+  Unit* units = reinterpret_cast<Unit*>(stage.data() + o_units);
+  NodeDev* const d_nodes = reinterpret_cast<NodeDev*>(base + o_nodes);
+  CountPtrs counts{};
   for (uint32_t n = 0; n < N; ++n) {
     uint8_t* nb = base + o_state + L.per_node * n;
-    NodeDev& nd = nodes[n];
-    std::memset(&nd, 0, sizeof nd);
+    NodeDev& nd = nodes[n];  // zero so far
     const igs_static_output& o = outs[n];
     nd.node = n;
     nd.N = N;
@@ -229,55 +278,49 @@ extern "C" int igs_lower_static(const igs_config* cfg, const igs_static_buffer* 
     nd.boxes = o.boxes;
     nd.binds = o.binds;
     nd.diags = o.diags;
-    units[n].node = reinterpret_cast<NodeDev*>(base + o_nodes) + n;
+    units[n].node = d_nodes + n;
     units[n].prog = reinterpret_cast<ProgDev*>(base + o_prog);
+    counts.p[n] = o.counts;
   }
-  ProgDev pg;
+  ProgDev pg{};
   pg.items = reinterpret_cast<const Item*>(base + o_items);
   pg.tasks = reinterpret_cast<const igs_task*>(base + o_tasks);
   pg.bufs = reinterpret_cast<const BufDesc*>(base + o_bufs);
   pg.n_items = reinterpret_cast<volatile uint32_t*>(base + o_nitems);
+  std::memcpy(stage.data() + o_prog, &pg, sizeof pg);
   const uint32_t n_items = (uint32_t)items.size();
-  const igs_instruction i0{0, IGS_EPOCH, NONE, NONE, NONE, NONE, NONE, 0, 0, 0, 0};
-  // the array keeps the previous call's contents: reset what must start at zero
+  std::memcpy(stage.data() + o_nitems, &n_items, sizeof n_items);
+  if (n_items) std::memcpy(stage.data() + o_items, items.data(), sizeof(Item) * n_items);
+  if (num_tasks) std::memcpy(stage.data() + o_tasks, tasks, sizeof(igs_task) * num_tasks);
+  if (num_buffers) std::memcpy(stage.data() + o_bufs, bd.data(), sizeof(BufDesc) * num_buffers);
 #define CKS(x)                          \
   do {                                  \
     if ((x) != cudaSuccess) return IGS_ERR_CUDA; \
   } while (0)
-  CKS(cudaMemcpyAsync(base + o_nodes, nodes.data(), sizeof(NodeDev) * N, cudaMemcpyHostToDevice, stream));
-  CKS(cudaMemcpyAsync(base + o_units, units.data(), sizeof(Unit) * N, cudaMemcpyHostToDevice, stream));
-  CKS(cudaMemcpyAsync(base + o_prog, &pg, sizeof pg, cudaMemcpyHostToDevice, stream));
-  CKS(cudaMemcpyAsync(base + o_nitems, &n_items, sizeof n_items, cudaMemcpyHostToDevice, stream));
-  if (n_items) CKS(cudaMemcpyAsync(base + o_items, items.data(), sizeof(Item) * n_items, cudaMemcpyHostToDevice, stream));
-  if (num_tasks) CKS(cudaMemcpyAsync(base + o_tasks, tasks, sizeof(igs_task) * num_tasks, cudaMemcpyHostToDevice, stream));
-  if (num_buffers) CKS(cudaMemcpyAsync(base + o_bufs, bd.data(), sizeof(BufDesc) * num_buffers, cudaMemcpyHostToDevice, stream));
-  for (uint32_t n = 0; n < N; ++n) {
-    uint8_t* nb = base + o_state + L.per_node * n;
-    CKS(cudaMemsetAsync(nb + L.o_desc, 0, 4 * igs::kDesc * (2 * kBuffers + 2 * kSlots), stream));
-    CKS(cudaMemsetAsync(nb + L.o_succ, 0, 1, stream));
-    CKS(cudaMemcpyAsync(nb + L.o_free, slots.data(), 4 * kSlots, cudaMemcpyHostToDevice, stream));
-    CKS(cudaMemcpyAsync(outs[n].instrs, &i0, sizeof i0, cudaMemcpyHostToDevice, stream));
+  uint32_t result[64];  // {status, rejected tasks} per node
+  // Each node is lowered by its block's helper and front
+  // warps together (one warp per node took 15.4 ms for 28 wave tasks on 4 x 4
+  // devices in 64 chunks, the shared form 7.7 ms). Their staging and the
+  // slabs they place may run out where a single warp's do not, so whatever
+  // does not come out well is lowered again, from the start, by one warp.
+  for (int helped = N <= kHelpedNodes ? 1 : 0; helped >= 0; --helped) {
+    for (uint32_t n = 0; n < N; ++n)
+      nodes[n].helper_scratch = helped ? reinterpret_cast<uint32_t*>(helpers + kHelperBytes * n) : nullptr;
+    CKS(cudaMemcpyAsync(base, stage.data(), o_state, cudaMemcpyHostToDevice, stream));
+    static_init<<<N, 128, 0, stream>>>(d_nodes);
+    if (igs_launch_lower(reinterpret_cast<const Unit*>(base + o_units), N, NONE, stream, false, nullptr, helped != 0))
+      return IGS_ERR_CUDA;
+    static_counts<<<1, 32, 0, stream>>>(d_nodes, N, counts, reinterpret_cast<uint32_t*>(base + o_result));
+    CKS(cudaGetLastError());
+    CKS(cudaMemcpyAsync(result, base + o_result, 8 * N, cudaMemcpyDeviceToHost, stream));
+    CKS(cudaStreamSynchronize(stream));
+    bool ok = true;
+    for (uint32_t n = 0; n < N; ++n) ok = ok && result[2 * n] == ST_OK;
+    if (ok) break;
   }
-  if (igs_launch_lower(reinterpret_cast<const Unit*>(base + o_units), N, NONE, stream)) return IGS_ERR_CUDA;
-  // counts and status of every node into the caller's device words
-  for (uint32_t n = 0; n < N; ++n) {
-    const NodeDev* nd = reinterpret_cast<const NodeDev*>(base + o_nodes) + n;
-    uint32_t* cnt = outs[n].counts;
-    CKS(cudaMemcpyAsync(cnt + 0, &nd->n_instr, 4, cudaMemcpyDeviceToDevice, stream));
-    CKS(cudaMemcpyAsync(cnt + 1, &nd->n_edge, 4, cudaMemcpyDeviceToDevice, stream));
-    CKS(cudaMemcpyAsync(cnt + 2, &nd->n_box, 4, cudaMemcpyDeviceToDevice, stream));
-    CKS(cudaMemcpyAsync(cnt + 3, &nd->n_bind, 4, cudaMemcpyDeviceToDevice, stream));
-    CKS(cudaMemcpyAsync(cnt + 4, &nd->n_diag, 4, cudaMemcpyDeviceToDevice, stream));
-    CKS(cudaMemcpyAsync(cnt + 5, &nd->status, 4, cudaMemcpyDeviceToDevice, stream));
-  }
-  // tasks rejected for overlapping writes (Sec. 4.4), counted per node
-  uint32_t rej[32];
-  for (uint32_t n = 0; n < N; ++n)
-    CKS(cudaMemcpyAsync(&rej[n], &(reinterpret_cast<const NodeDev*>(base + o_nodes) + n)->n_rej, 4,
-                        cudaMemcpyDeviceToHost, stream));
-  CKS(cudaStreamSynchronize(stream));
 #undef CKS
+  // tasks rejected for overlapping writes (Sec. 4.4), counted per node
   for (uint32_t n = 0; n < N; ++n)
-    if (rej[n]) return IGS_ERR_OVERLAPPING_WRITE;
+    if (result[2 * n + 1]) return IGS_ERR_OVERLAPPING_WRITE;
   return IGS_OK;
 }
