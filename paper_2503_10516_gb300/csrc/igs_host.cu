@@ -1003,9 +1003,9 @@ struct FlowBuild {
   // appends a copy job to node F (the last node added); tiles counts units so far
   void add_copy(uint32_t F, CopyJob J) {
     FlowNode& f = nodes[F];
+    split_copy(J, kCopyUnit);
     J.unit_begin = f.tiles;
-    const uint64_t segs = (J.extent[2] + J.seg_bytes - 1) / J.seg_bytes;
-    f.tiles += (uint32_t)((uint64_t)J.extent[0] * J.extent[1] * segs);
+    f.tiles += (uint32_t)copy_units(J);
     copies.push_back(J);
     f.count++;
   }
@@ -1073,19 +1073,11 @@ bool make_copy_job(const uint8_t* src, const uint32_t slo[3], const uint32_t shi
   // very long runs are split into rows of at most 1 GiB to keep 32-bit lengths
   J.extent[2] = (uint32_t)std::min<uint64_t>(run, 1ull << 30);
   if (run > (1ull << 30)) return false;
-  J.seg_bytes = 64 * 1024;
   return true;
 }
 
-// Appends a copy job to level L's box-copy launch (its work units follow the level's earlier jobs).
-void add_copy(Pending& p, uint32_t L, const CopyJob& J) {
-  LevelWork& w = p.at(L);
-  CopyJob j = J;
-  j.unit_begin = w.copy_units;
-  const uint64_t segs = (j.extent[2] + j.seg_bytes - 1) / j.seg_bytes;
-  w.copy_units += (uint64_t)j.extent[0] * j.extent[1] * segs;
-  w.copies.push_back(j);
-}
+// Appends a copy job to level L's box-copy launch.
+void add_copy(Pending& p, uint32_t L, const CopyJob& J) { p.at(L).copies.push_back(J); }
 
 void add_kernel(Pending& p, uint32_t L, KernelJob J, uint64_t items, bool stencil) {
   LevelWork& w = p.at(L);
@@ -1214,6 +1206,7 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
   for (size_t L = 0; L < p.levels.size(); ++L) {
     LevelWork& w = p.levels[L];
     co[L] = nc;
+    w.copy_units = place_copies(w.copies.data(), w.copies.size());
     std::copy(w.copies.begin(), w.copies.end(), c->h_cjobs[k] + nc);
     nc += w.copies.size();
     ko[L] = nk;
@@ -2110,7 +2103,6 @@ extern "C" int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream) 
   igs_ctx* c = nullptr;
   if (!jobs && n) return IGS_ERR_INVALID_ARG;
   std::vector<CopyJob> v;
-  uint64_t units = 0;
   for (uint32_t i = 0; i < n; ++i) {
     const igs_copy_job& j = jobs[i];
     CopyJob J{};
@@ -2121,11 +2113,15 @@ extern "C" int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream) 
     if (!make_copy_job(static_cast<const uint8_t*>(j.src), j.src_box.lo, j.src_box.hi, static_cast<uint8_t*>(j.dst),
                        j.dst_box.lo, j.dst_box.hi, j.box, j.elem_size, J))
       continue;
-    J.unit_begin = units;
-    units += (uint64_t)J.extent[0] * J.extent[1] * ((J.extent[2] + J.seg_bytes - 1) / J.seg_bytes);
     v.push_back(J);
   }
   if (v.empty()) return IGS_OK;
+  const uint64_t units = place_copies(v.data(), v.size());
+  if (v.size() <= kCopyFewJobs) {
+    if (igs_launch_copies_few(v.data(), (uint32_t)v.size(), units, stream)) return IGS_ERR_CUDA;
+    CK(cudaStreamSynchronize((cudaStream_t)stream));
+    return IGS_OK;
+  }
   static thread_local CopyJob* d_jobs = nullptr;
   static thread_local size_t cap = 0;
   if (v.size() > cap) {

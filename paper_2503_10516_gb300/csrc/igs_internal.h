@@ -148,15 +148,74 @@ struct ServeSlot {
   volatile uint32_t state, done, status, exit, busy, pad;
 };
 
-// Box-copy work descriptor (device side).
+// Box-copy work descriptor (device side): extent[0] x extent[1] rows of
+// extent[2] contiguous bytes.
 struct CopyJob {
   const uint8_t* src;
   uint8_t* dst;
   uint64_t src_stride[2], dst_stride[2];  // bytes per step of dim 0 / dim 1 (after collapsing)
   uint32_t extent[3];                     // rows0, rows1, contiguous bytes per row
-  uint32_t seg_bytes;                     // bytes per work unit along the row
+  uint32_t seg_bytes;                     // bytes of a row per work unit (units of one row)
+  uint32_t rows_unit;                     // rows of dim 1 per work unit
+  uint32_t gran;                          // short rows: the largest power of two (<= 16) all addresses and the run share
   uint64_t unit_begin;                    // prefix of work units
 };
+
+// Rows shorter than this (one round of a warp's vectors) are copied element by
+// element, a unit's rows side by side; longer ones by a warp each, or by the
+// warps of a block together.
+constexpr uint32_t kCopyShortRow = 512;
+constexpr uint32_t kCopyWarps = 8;  // warps of a copying block
+// Jobs that travel in the kernel's parameters (4 KB).
+constexpr uint32_t kCopyFewJobs = 44;
+
+inline uint64_t copy_units(const CopyJob& j) {
+  return (uint64_t)j.extent[0] * ((j.extent[1] - 1) / j.rows_unit + 1) *
+         ((j.extent[2] + j.seg_bytes - 1) / j.seg_bytes);
+}
+
+// Splits a job into work units of about `unit` bytes (a power of two).
+constexpr uint32_t kCopyUnit = 64 * 1024;
+inline void split_copy(CopyJob& j, uint32_t unit) {
+  const uint64_t run = j.extent[2];
+  uint64_t mix = (uint64_t)reinterpret_cast<uintptr_t>(j.src) | (uint64_t)reinterpret_cast<uintptr_t>(j.dst) | run | 16;
+  if (j.extent[0] > 1) mix |= j.src_stride[0] | j.dst_stride[0];
+  if (j.extent[1] > 1) mix |= j.src_stride[1] | j.dst_stride[1];
+  j.gran = (uint32_t)(mix & (~mix + 1));
+  // units take rows of dim 1: the longer of the two, where dim 1 does not fill a unit
+  if (j.extent[0] > j.extent[1] && j.extent[1] * run < unit) {
+    uint32_t e = j.extent[0];
+    j.extent[0] = j.extent[1];
+    j.extent[1] = e;
+    uint64_t t = j.src_stride[0];
+    j.src_stride[0] = j.src_stride[1];
+    j.src_stride[1] = t;
+    t = j.dst_stride[0];
+    j.dst_stride[0] = j.dst_stride[1];
+    j.dst_stride[1] = t;
+  }
+  j.rows_unit = 1;
+  if (run < kCopyShortRow) j.rows_unit = (uint32_t)(unit / run);  // at most 2^16 elements
+  else if (kCopyWarps * run <= 4 * unit) j.rows_unit = kCopyWarps;  // else the warps share a piece of one row
+  j.seg_bytes = unit;
+}
+
+// Splits the jobs of one launch and numbers their units: units of 4 to 64 KB,
+// about four per SM, so that a small copy is spread over the chip and a large
+// one pays for few units (5 copies of 7 MB: 29 us in 8 KB units, 22 us in 32
+// KB units). Returns the number of units.
+inline uint64_t place_copies(CopyJob* jobs, size_t n) {
+  uint64_t total = 0, units = 0;
+  for (size_t i = 0; i < n; ++i) total += (uint64_t)jobs[i].extent[0] * jobs[i].extent[1] * jobs[i].extent[2];
+  uint32_t unit = kCopyUnit;
+  while (unit > 4096 && total / unit < 608) unit >>= 1;
+  for (size_t i = 0; i < n; ++i) {
+    split_copy(jobs[i], unit);
+    jobs[i].unit_begin = units;
+    units += copy_units(jobs[i]);
+  }
+  return units;
+}
 
 }  // namespace igs
 
@@ -179,3 +238,5 @@ int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_
 // warp stays idle for idle_polls polls (about 2 us each).
 int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t* stop, uint64_t idle_polls, void* stream);
 int igs_launch_copies(const igs::CopyJob* jobs_dev, uint32_t n_jobs, uint64_t n_units, void* stream);
+// The same for at most kCopyFewJobs jobs in host memory.
+int igs_launch_copies_few(const igs::CopyJob* jobs, uint32_t n_jobs, uint64_t n_units, void* stream);

@@ -103,3 +103,50 @@ def test_stencil_strips(shape, chunks, kind, executor):
         got = c.read_buffer(i, (0, 0, 0), (*shape, 1), 4).view(np.float32).reshape(shape)
         assert np.array_equal(got, w), (shape, i)
     c.close()
+
+
+def _copy_case(torch, rng, n_jobs, elem, ext, pads, offs):
+    """n_jobs copies of a box of extent ext between allocations that are wider
+    by pads (source, destination) per dimension, their first bytes off by offs."""
+    from paper_2503_10516_gb300 import igs
+    jobs, want, keep = (igs.CopyJob * n_jobs)(), [], []
+    for j in range(n_jobs):
+        arrs = []
+        for k in range(2):
+            shape = [e + p for e, p in zip(ext, pads[k])]
+            host = rng.integers(0, 256, size=int(np.prod(shape)) * elem, dtype=np.uint8)
+            dev = torch.zeros(len(host) + 16, dtype=torch.uint8, device="cuda")
+            dev[offs[k]:offs[k] + len(host)] = torch.from_numpy(host).cuda()
+            arrs.append((host.reshape(*shape, elem), dev, shape))
+        (src, sdev, ss), (dst, ddev, ds) = arrs
+        jobs[j].src, jobs[j].dst, jobs[j].elem_size = sdev.data_ptr() + offs[0], ddev.data_ptr() + offs[1], elem
+        for box, shape, pad in ((jobs[j].src_box, ss, pads[0]), (jobs[j].dst_box, ds, pads[1]), (jobs[j].box, ext, (0,) * 3)):
+            lo = [100 - p // 2 for p in pad]
+            box.lo[:], box.hi[:] = lo, [v + s for v, s in zip(lo, shape)]
+        at = [tuple(slice(p // 2, p // 2 + e) for p, e in zip(pad, ext)) for pad in pads]
+        dst[at[1]] = src[at[0]]
+        keep.append((sdev, ddev))
+        want.append(dst.reshape(-1))
+    r = igs.lib().igs_box_copy(jobs, n_jobs, torch.cuda.current_stream().cuda_stream)
+    assert r == igs.IGS_OK
+    for (_, ddev), w in zip(keep, want):
+        got = ddev.cpu().numpy()
+        assert np.array_equal(got[offs[1]:offs[1] + len(w)], w)
+        assert not got[:offs[1]].any() and not got[offs[1] + len(w):].any()
+
+
+@pytest.mark.parametrize("elem", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("run", [1, 15, 16, 31, 47, 511, 512, 513, 4095, 4096, 8191, 8193, 65537])
+def test_box_copy_rows(elem, run):
+    """Rows of about `run` bytes: around the short rows, a row per warp, a
+    span per warp and several pieces per row, at every alignment of the two
+    sides, rows side by side in dimension 0 or 1, few and many jobs."""
+    import torch
+    rng = np.random.default_rng(run)
+    cols = max(1, run // elem)
+    cases = [(1, (1, 1, cols), ((0, 0, 0), (0, 0, 0)), (0, 0)), (1, (1, 9, cols), ((0, 0, 0), (0, 0, 3)), (0, 0)),
+             (3, (5, 3, cols), ((0, 1, 2), (1, 0, 5)), (0, 0)), (5, (33, 2, cols), ((2, 0, 0), (0, 2, 7)), (4, 0)),
+             (1, (2, 17, cols), ((0, 0, 4), (0, 3, 8)), (0, 4)), (1, (3, 7, cols), ((0, 0, 1), (0, 0, 4)), (1, 6)),
+             (44, (1, 2, cols), ((0, 0, 1), (0, 0, 0)), (0, 0)), (45, (2, 1, cols), ((0, 0, 0), (0, 1, 1)), (8, 8))]
+    for c in cases:
+        _copy_case(torch, rng, *c[:1], elem, *c[1:])
