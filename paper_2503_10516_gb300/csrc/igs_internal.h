@@ -46,6 +46,7 @@ struct Table {
 // Warps that share parts of a node's lowering (warp 0 and up to 7 helpers),
 // and the scratch tables of each helper.
 constexpr uint32_t kMaxWorkers = 8;
+constexpr uint32_t kQueueWarps = 8;  // of a work-queue block, at most
 constexpr uint32_t kHelperTables = 12;
 // Scratch sets in a node's helper scratch: one per worker, plus one for the
 // front warp that runs push / await push ahead of warp 0 (pipelined launches).
@@ -220,11 +221,19 @@ inline uint64_t place_copies(CopyJob* jobs, size_t n) {
 }  // namespace igs
 
 // Device entry points implemented in the .cu translation units.
-// Persistent blocks of `warps` warps (1..kMaxWorkers) pulling units from a
+// Persistent blocks of `warps` warps (1..kQueueWarps) pulling units from a
 // device work queue (*head, zero before the launch) in the order order_dev
 // (null = index order); extra warps help nodes that have helper scratch.
 int igs_launch_lower_queue(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                            uint32_t blocks, uint32_t warps, void* stream);
+// Blocks with helper and front warps and scratch of their own (each
+// igs_lower_pool_words words of scratch_dev; cap_scratch and front_cap: the
+// largest scratch and push / await table capacities among the units' nodes),
+// pulling units in the order order_dev.
+size_t igs_lower_pool_words(uint32_t cap_scratch, uint32_t front_cap);
+int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
+                          uint32_t blocks, uint32_t* scratch_dev, uint32_t cap_scratch, uint32_t front_cap,
+                          void* stream);
 // One block per unit.
 // reserve: each unit's block also holds most of its SM's registers, keeping
 // other kernels off the SMs that lower (used while the executor runs concurrently).

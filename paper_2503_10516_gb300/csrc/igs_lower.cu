@@ -2133,6 +2133,8 @@ struct Pipe {
   volatile uint32_t rejected[kPipeDepth];  // the slot's task had overlapping writes
   volatile uint32_t n[kPipeDepth];         // push / await entries staged in the slot
   uint32_t begin, end;                     // the items this launch lowers
+  uint32_t* qr;                            // the slots' tables, kPipeDepth of qr_cap entries
+  uint32_t qr_cap;
 };
 
 struct BlockShared {
@@ -2141,6 +2143,9 @@ struct BlockShared {
   WorkJob job;
   uint32_t piped;
   Pipe pipe;
+  // blocks of a batch with helper scratch of their own: the unit being
+  // lowered, and whether its node uses that scratch
+  uint32_t unit, lent;
 };
 
 __device__ __forceinline__ void worker_bar(uint32_t workers) {
@@ -2187,6 +2192,19 @@ __device__ bool run_shared(Ctx& c, BlockShared& sh, uint32_t cmd, F share0) {
     c.err_info = sh.err_info;
   }
   return c.err == ST_OK;
+}
+
+// Whether a phase that only plans (no table has changed) failed for want of
+// room in a stage or scratch table: then, in blocks that lend their scratch
+// (calls that one warp used to serve), the failure is cleared, and the caller
+// takes the single-warp path, which stages nothing.
+__device__ bool plan_overflowed(Ctx& c) {
+  if (c.err != ST_CAPACITY || (c.err_info >> 24) != (uint32_t)CAP_TABLE ||
+      !static_cast<BlockShared*>(c.block)->lent)
+    return false;
+  c.err = ST_OK;
+  c.err_info = 0;
+  return true;
 }
 
 // Per buffer: missing_m = reads of node m's chunks not replicated on m; this
@@ -2348,7 +2366,7 @@ __device__ __noinline__ void a3_task(Ctx& c, const igs_task& t, uint32_t seq, co
       if (t.acc[a].buffer == b) done |= 1u << a;
     bufs[nbuf++] = b;
   }
-  if (c.block && c.workers > 1 && c.nd->helper_scratch && nbuf > 1) {
+  if (c.block && c.workers > 1 && c.nd->helper_scratch && nbuf > 1 && !static_cast<BlockShared*>(c.block)->lent) {
     BlockShared& sh = *static_cast<BlockShared*>(c.block);
     WorkJob& j = sh.job;
     Table& OUT0 = c.s[S_T5];
@@ -2984,7 +3002,8 @@ __device__ __noinline__ void p4_apply(Ctx& c, const WorkJob& j, uint32_t w) {
 // Warp 0: plan with the helpers; then, in consumer order, the warnings of
 // uninitialized reads, the copies' final ids and the capacity checks; then
 // the append (warp 0) beside the table updates (helpers).
-__device__ __noinline__ void p4_parallel(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, Table& PC,
+// Returns false (nothing done) when the plan did not fit the stages.
+__device__ __noinline__ bool p4_parallel(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, Table& PC,
                                          uint32_t na, bool states_later) {
   BlockShared& sh = *static_cast<BlockShared*>(c.block);
   WorkJob& j = sh.job;
@@ -3004,7 +3023,7 @@ __device__ __noinline__ void p4_parallel(Ctx& c, const igs_task& t, uint32_t seq
     j.n_live = c.n_live;
     j.p4_states_later = states_later ? 1u : 0u;
   }
-  if (!run_shared(c, sh, CMD_P4, [&]() { p4_share(c, j, 0); })) return;
+  if (!run_shared(c, sh, CMD_P4, [&]() { p4_share(c, j, 0); })) return !plan_overflowed(c);
   NodeDev* nd = c.nd;
   uint32_t next = c.n_instr, n_edge = 0, n_box = 0;
   p4_each(PC, 3u, NONE, [&](uint32_t k) -> bool {
@@ -3036,16 +3055,16 @@ __device__ __noinline__ void p4_parallel(Ctx& c, const igs_task& t, uint32_t seq
     next += cnt;
     return true;
   });
-  if (c.err) return;
+  if (c.err) return true;
   n_edge = warp_sum(n_edge);
   n_box = warp_sum(n_box);
   if (next > nd->cap_instr || c.n_edge + n_edge > nd->cap_edge) {
     fail_cap(c, CAP_EDGE, nd->cap_edge);
-    return;
+    return true;
   }
   if (c.n_box + n_box > nd->cap_box) {
     fail_cap(c, CAP_BOX, nd->cap_box);
-    return;
+    return true;
   }
   __syncwarp();
   // with a planned kernel phase to follow, about half of the up-to-date bits
@@ -3083,6 +3102,7 @@ __device__ __noinline__ void p4_parallel(Ctx& c, const igs_task& t, uint32_t seq
       return true;
     });
   });
+  return true;
 }
 
 // a9 over every table: with helper warps, shared by the workers.
@@ -3460,8 +3480,9 @@ __device__ __noinline__ void p5_finish(Ctx& c, const WorkJob& j, uint32_t w) {
 }
 
 // Warp 0: kernel ids, planners and owners; plan with the helpers; every
-// local kernel's place in the graph; finish with the helpers.
-__device__ __noinline__ void p5_planned(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP,
+// local kernel's place in the graph; finish with the helpers. Returns false
+// (no kernel emitted) when the plan did not fit the stages.
+__device__ __noinline__ bool p5_planned(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP,
                                         Table& AL, uint32_t na, bool p4_states_pending) {
   BlockShared& sh = *static_cast<BlockShared*>(c.block);
   NodeDev* nd = c.nd;
@@ -3518,7 +3539,7 @@ __device__ __noinline__ void p5_planned(Ctx& c, const igs_task& t, uint32_t seq,
     j.stage0 = reinterpret_cast<igs_edge*>(c.s[S_T0].base);
     j.p4_states_later = p4_states_pending ? 1u : 0u;  // j.PC still holds the coherence consumers
   }
-  if (!run_shared(c, sh, CMD_P5_PLAN, [&]() { p5_plan(c, sh.job, 0); })) return;
+  if (!run_shared(c, sh, CMD_P5_PLAN, [&]() { p5_plan(c, sh.job, 0); })) return !plan_overflowed(c);
   // places in chunk order; the first kernel that would overflow a capacity
   // fails as in the single-warp path (edges and records, then boxes, then
   // bindings)
@@ -3553,14 +3574,15 @@ __device__ __noinline__ void p5_planned(Ctx& c, const igs_task& t, uint32_t seq,
     if (bad_kind == 1) fail_cap(c, CAP_EDGE, nd->cap_edge);
     else if (bad_kind == 2) fail_cap(c, CAP_BOX, nd->cap_box);
     else fail_cap(c, CAP_BIND, nd->cap_bind);
-    return;
+    return true;
   }
   __syncwarp();
-  if (!run_shared(c, sh, CMD_P5_FINISH, [&]() { p5_finish(c, sh.job, 0); })) return;
+  if (!run_shared(c, sh, CMD_P5_FINISH, [&]() { p5_finish(c, sh.job, 0); })) return true;
   c.n_instr += n_k;
   c.n_edge = n_edge;
   c.n_box = n_box;
   c.n_bind = n_bind;
+  return true;
 }
 
 // P2 of task item (qr entries [qs, qe)): per (buffer, target) in ascending
@@ -3812,6 +3834,28 @@ __device__ __noinline__ void p3_plan(Ctx& c, WorkJob& j, uint32_t w) {
   c.snap_alloc = NONE;
 }
 
+// P3 of a task (qr entries [qs, qe)) by this warp alone.
+__device__ __noinline__ void p3_awaits(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP,
+                                       uint32_t qs, uint32_t qe) {
+  for (uint32_t g0 = qs; g0 < qe;) {
+    uint32_t g1 = g0;
+    while (g1 < qe && t_v(c.qr, 0, g1) == t_v(c.qr, 0, g0)) ++g1;
+    const uint32_t kind = t_v(c.qr, 0, g0);
+    if (kind != 1) {
+      g0 = g1 + (kind == 0 ? 1 : 0);
+      continue;
+    }
+    const uint32_t dst = find_alloc(c, t_v(c.qr, 1, g0), 1, t_box(c.qr, g1));
+    if (dst == NONE) {
+      fail_internal(c, 7);
+      return;
+    }
+    p3_group(c, t, seq, CH, MP, c.qr, g0, g1, dst);
+    if (c.err) return;
+    g0 = g1 + 1;
+  }
+}
+
 __device__ __noinline__ bool p23_parallel(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP,
                                           uint32_t qs, uint32_t qe) {
   if (!c.block || c.workers < 2 || !c.nd->helper_scratch || c.nd->stage_d2d) return false;
@@ -3877,7 +3921,15 @@ __device__ __noinline__ bool p23_parallel(Ctx& c, const igs_task& t, uint32_t se
     j.workers = c.workers;
     j.p3_n = n;
   }
-  if (!run_shared(c, sh, CMD_P3, [&]() { p2_pushes(c, seq, qs, qe); })) return true;
+  uint32_t own = ST_OK;
+  if (!run_shared(c, sh, CMD_P3, [&]() {
+        p2_pushes(c, seq, qs, qe);
+        own = c.err;
+      })) {
+    // the pushes are done: awaits whose plans did not fit follow them
+    if (own == ST_OK && plan_overflowed(c)) p3_awaits(c, t, seq, CH, MP, qs, qe);
+    return true;
+  }
   // the planned instructions in group order, each with the single-warp
   // path's table updates
   for (uint32_t gi = 0; gi < n && !c.err; ++gi) {
@@ -3995,23 +4047,7 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
     p2_pushes(c, seq, qs, qe);
     if (c.err) return;
     pt_lap(pt, c, PH_P2);
-    for (uint32_t g0 = qs; g0 < qe;) {
-      uint32_t g1 = g0;
-      while (g1 < qe && t_v(c.qr, 0, g1) == t_v(c.qr, 0, g0)) ++g1;
-      const uint32_t kind = t_v(c.qr, 0, g0);
-      if (kind != 1) {
-        g0 = g1 + (kind == 0 ? 1 : 0);
-        continue;
-      }
-      const uint32_t dst = find_alloc(c, t_v(c.qr, 1, g0), 1, t_box(c.qr, g1));
-      if (dst == NONE) {
-        fail_internal(c, 7);
-        return;
-      }
-      p3_group(c, t, seq, CH, MP, c.qr, g0, g1, dst);
-      if (c.err) return;
-      g0 = g1 + 1;
-    }
+    p3_awaits(c, t, seq, CH, MP, qs, qe);
   }
   if (c.err) return;
   pt_lap(pt, c, PH_P3);
@@ -4091,9 +4127,10 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
   // a planned kernel phase sets the coherence copies' up-to-date bits
   const bool p5_shared = c.block && c.workers > 2 && c.nd->helper_scratch && p5_plannable(t);
   if (multi) {
-    p4_parallel(c, t, seq, CH, PC, na, p5_shared);
+    multi = p4_parallel(c, t, seq, CH, PC, na, p5_shared);
     if (c.err) return;
-  } else {
+  }
+  if (!multi) {
     for (uint32_t k = 0; k < PC.n; ++k) {
       if (!t_key(PC, k)) continue;
       if (!p4_consumer(c, t, seq, CH, PC, k, na, true)) return;
@@ -4134,13 +4171,17 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
     AL.n = total;
     __syncwarp();
   }
-  bool planned = false;
+  bool planned = false, done = false;
   if (c.block && c.workers > 1 && c.nd->helper_scratch) {
-    planned = p5_plannable(t);
-    if (planned) p5_planned(c, t, seq, CH, MP, AL, na, multi && p5_shared);
-    else p5_parallel(c, t, seq, CH, MP, AL, na);
+    if (p5_plannable(t)) {
+      done = planned = p5_planned(c, t, seq, CH, MP, AL, na, multi && p5_shared);
+    } else if (!static_cast<BlockShared*>(c.block)->lent) {
+      p5_parallel(c, t, seq, CH, MP, AL, na);
+      done = true;
+    }
     if (c.err) return;
-  } else {
+  }
+  if (!done) {
     for (uint32_t slot = 0; slot < CH.n; ++slot) {
       if (t_v(CH, 0, slot) != c.node) continue;
       const uint32_t mem = t_v(CH, 1, slot);
@@ -4371,7 +4412,7 @@ __device__ void own_create(Ctx& c, const Item& it) {
 __device__ void pipe_take(Ctx& c, uint32_t item) {
   const uint32_t slot = item % kPipeDepth, cnt = c.pipe->n[slot];
   if (cnt == 0) return;
-  const uint32_t* src = helper_table(c.nd, kFrontWarp, 8 + slot);
+  const uint32_t* src = c.pipe->qr + (size_t)slot * c.pipe->qr_cap * F_COUNT;
   const uint32_t first = __shfl_sync(FULL, t_claim_n(c, c.qr, laneid() == 0 ? cnt : 0u), 0);  // lane 0's slot
   if (c.err) return;
   const uint4* s4 = reinterpret_cast<const uint4*>(src);
@@ -4611,7 +4652,7 @@ __device__ void front_loop(BlockShared& sh, const Unit u) {
   for (uint32_t i = P.begin; i < P.end && f.err == ST_OK; ++i) {
     if (!pipe_wait(f, P, [&]() { return i - P.back_done < kPipeDepth; }, 256)) break;
     const uint32_t slot = i % kPipeDepth;
-    f.qr = scratch_table(helper_table(u.node, kFrontWarp, 8 + slot), cap);
+    f.qr = scratch_table(P.qr + (size_t)slot * P.qr_cap * F_COUNT, P.qr_cap);
     uint32_t rejected = 0;
     const Item it = f.pg->items[i];
     if (it.kind == IT_CREATE) {
@@ -4714,41 +4755,38 @@ __device__ void lower_unit(const Unit* units, uint32_t n_units, uint32_t max_ite
 // SM's registers, so no block of another kernel (the executor's copies and
 // kernels running concurrently) shares the SM, its issue slots or its L1.
 constexpr uint32_t kReserveThreads = 512;
-__global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* units, uint32_t n_units, uint32_t max_items,
-                                                               volatile uint32_t* progress) {
-  __shared__ BlockShared sh;
+// Thread 0: a block's shared state before it lowers unit u: a front warp when
+// the block has one, the node has its scratch set and the launch lowers
+// several items.
+__device__ void unit_begin(BlockShared& sh, const Unit& u, uint32_t warps, uint32_t max_items) {
+  sh.lock = 0;
+  sh.cmd = CMD_NONE;
+  sh.err = ST_OK;
+  sh.piped = 0;
+  const NodeDev* nd = u.node;
+  if (warps <= kFrontWarp || !nd->helper_scratch || nd->status != ST_OK) return;
+  const uint32_t cur = nd->cursor, avail = *u.prog->n_items;
+  uint32_t end = avail;
+  if (max_items != NONE && cur + max_items < end) end = cur + max_items;
+  if (end <= cur || end - cur < kPipeMinItems) return;
+  sh.piped = 1;
+  sh.pipe.begin = cur;
+  sh.pipe.end = end;
+  sh.pipe.front_done = cur;
+  sh.pipe.back_done = cur;
+  sh.pipe.abort = 0;
+  sh.pipe.err = ST_OK;
+  sh.pipe.err_info = 0;
+  sh.pipe.qr = helper_table(nd, kFrontWarp, 8);
+  sh.pipe.qr_cap = nd->cap_scratch;
+}
+// The block's warps in their roles for unit w, after unit_begin and a barrier.
+__device__ void unit_body(BlockShared& sh, const Unit* units, uint32_t n_units, uint32_t w, uint32_t max_items,
+                          volatile uint32_t* progress) {
   const uint32_t warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const uint32_t workers = nw < kMaxWorkers ? nw : kMaxWorkers;
-  if (threadIdx.x == 0) {
-    sh.lock = 0;
-    sh.cmd = CMD_NONE;
-    sh.err = ST_OK;
-    sh.piped = 0;
-    // a front warp when the block has one, the node has its scratch set and
-    // the launch lowers several items
-    if (nw > kFrontWarp && blockIdx.x < n_units) {
-      const Unit u = units[blockIdx.x];
-      const NodeDev* nd = u.node;
-      if (nd->helper_scratch && nd->status == ST_OK) {
-        const uint32_t cur = nd->cursor, avail = *u.prog->n_items;
-        uint32_t end = avail;
-        if (max_items != NONE && cur + max_items < end) end = cur + max_items;
-        if (end > cur && end - cur >= kPipeMinItems) {
-          sh.piped = 1;
-          sh.pipe.begin = cur;
-          sh.pipe.end = end;
-          sh.pipe.front_done = cur;
-          sh.pipe.back_done = cur;
-          sh.pipe.abort = 0;
-          sh.pipe.err = ST_OK;
-          sh.pipe.err_info = 0;
-        }
-      }
-    }
-  }
-  __syncthreads();
   if (warp == 0) {
-    lower_unit(units, n_units, max_items, blockIdx.x, progress, workers > 1 ? &sh : nullptr, workers,
+    lower_unit(units, n_units, max_items, w, progress, workers > 1 ? &sh : nullptr, workers,
                sh.piped ? &sh.pipe : nullptr);
     if (workers > 1) {
       if ((threadIdx.x & 31u) == 0) {
@@ -4761,9 +4799,52 @@ __global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* unit
   } else if (warp < workers) {
     helper_loop(sh, warp, workers);
   } else if (warp == kFrontWarp && sh.piped) {
-    front_loop(sh, units[blockIdx.x]);
+    front_loop(sh, units[w]);
   }
   __syncthreads();
+}
+
+__global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* units, uint32_t n_units, uint32_t max_items,
+                                                               volatile uint32_t* progress) {
+  __shared__ BlockShared sh;
+  if (threadIdx.x == 0) {
+    sh.lent = 0;
+    unit_begin(sh, units[blockIdx.x], blockDim.x >> 5, max_items);
+  }
+  __syncthreads();
+  unit_body(sh, units, n_units, blockIdx.x, max_items, progress);
+}
+
+// Batched lowering of few or uneven units, whose longest bounds the launch:
+// each resident block has helper scratch of its own (slot_words words, its
+// last kPipeDepth x front_cap entries the front warp's slots), lends it to the
+// node it lowers, and takes units longest first from *head.
+__global__ void __launch_bounds__(kReserveThreads) lower_pool_kernel(const Unit* units, uint32_t n_units,
+                                                                    const uint32_t* order, uint32_t* head,
+                                                                    uint32_t* scratch, size_t slot_words,
+                                                                    uint32_t front_cap) {
+  __shared__ BlockShared sh;
+  uint32_t* const mine = scratch + blockIdx.x * slot_words;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      const uint32_t i = atomicAdd(head, 1u);
+      sh.unit = i < n_units ? order[i] : NONE;
+      if (sh.unit != NONE) {
+        const Unit u = units[sh.unit];
+        sh.lent = u.node->helper_scratch == nullptr;
+        if (sh.lent) u.node->helper_scratch = mine;
+        unit_begin(sh, u, blockDim.x >> 5, NONE);
+        if (sh.lent) {
+          sh.pipe.qr = mine + slot_words - (size_t)kPipeDepth * front_cap * F_COUNT;
+          sh.pipe.qr_cap = front_cap;
+        }
+      }
+    }
+    __syncthreads();
+    if (sh.unit == NONE) break;
+    unit_body(sh, units, n_units, sh.unit, NONE, nullptr);
+    if (threadIdx.x == 0 && sh.lent) units[sh.unit].node->helper_scratch = nullptr;
+  }
 }
 
 // Batched lowering with a device work queue: the first warp of each
@@ -4772,7 +4853,7 @@ __global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* unit
 // unit is lowered. The block's other warps (if any) help with the shared
 // phases of units whose node has helper scratch, and wait at the block
 // barrier otherwise.
-__global__ void __launch_bounds__(32 * kMaxWorkers) lower_queue_kernel(const Unit* units, uint32_t n_units,
+__global__ void __launch_bounds__(32 * kQueueWarps) lower_queue_kernel(const Unit* units, uint32_t n_units,
                                                                       const uint32_t* order, uint32_t* head) {
   __shared__ BlockShared sh;
   const uint32_t warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -4781,6 +4862,7 @@ __global__ void __launch_bounds__(32 * kMaxWorkers) lower_queue_kernel(const Uni
     sh.lock = 0;
     sh.cmd = CMD_NONE;
     sh.err = ST_OK;
+    sh.lent = 0;
   }
   __syncthreads();
   if (warp == 0) {
@@ -4922,7 +5004,7 @@ int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t*
 
 int igs_launch_lower_queue(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                            uint32_t blocks, uint32_t warps, void* stream) {
-  if (warps < 1 || warps > igs::kMaxWorkers) return -1;
+  if (warps < 1 || warps > igs::kQueueWarps) return -1;
   if (n_units == 0) return 0;
   static bool carveout = false;
   if (!carveout) {
@@ -4930,6 +5012,25 @@ int igs_launch_lower_queue(const igs::Unit* units_dev, uint32_t n_units, const u
     carveout = true;
   }
   igs::lower_queue_kernel<<<blocks, 32 * warps, 0, (cudaStream_t)stream>>>(units_dev, n_units, order_dev, head_dev);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+size_t igs_lower_pool_words(uint32_t cap_scratch, uint32_t front_cap) {
+  return (size_t)igs::F_COUNT *
+         ((size_t)igs::kScratchSets * igs::kHelperTables * cap_scratch + (size_t)igs::kPipeDepth * front_cap);
+}
+
+int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
+                          uint32_t blocks, uint32_t* scratch_dev, uint32_t cap_scratch, uint32_t front_cap,
+                          void* stream) {
+  if (n_units == 0) return 0;
+  static bool carveout = false;
+  if (!carveout) {
+    cudaFuncSetAttribute(igs::lower_pool_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    carveout = true;
+  }
+  igs::lower_pool_kernel<<<blocks, 32 * (igs::kMaxWorkers + 1), 0, (cudaStream_t)stream>>>(
+      units_dev, n_units, order_dev, head_dev, scratch_dev, igs_lower_pool_words(cap_scratch, front_cap), front_cap);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
