@@ -448,18 +448,14 @@ __device__ __forceinline__ bool t_grow(Ctx& c, Table& t, uint32_t need) {
   return true;
 }
 
-// Claims one slot per predicated lane (all lanes call). NONE on overflow.
-__device__ __forceinline__ uint32_t t_claim(Ctx& c, Table& t, bool pred) {
-  const uint32_t m = __ballot_sync(FULL, pred);
-  const uint32_t slot = t.n + __popc(m & lanemask_lt());
-  const uint32_t nn = t.n + __popc(m);
-  if (nn > t.cap && !t_grow(c, t, nn)) return NONE;
-  t.n = nn;
-  t.live += __popc(m);
-  c.map_writes += __popc(m);
-  t_publish(c, t);
-  return pred ? slot : NONE;
+// Counts table entries read / written.
+__device__ __forceinline__ void count_reads(Ctx& c, uint32_t k) {
+  c.map_reads += k;
 }
+__device__ __forceinline__ void count_writes(Ctx& c, uint32_t k) {
+  c.map_writes += k;
+}
+
 // Claims one slot per predicated lane (all lanes call); false (every lane)
 // when the table could not grow.
 __device__ __forceinline__ bool t_claim_ok(Ctx& c, Table& t, bool pred, uint32_t& slot) {
@@ -469,8 +465,22 @@ __device__ __forceinline__ bool t_claim_ok(Ctx& c, Table& t, bool pred, uint32_t
   if (nn > t.cap && !t_grow(c, t, nn)) return false;
   t.n = nn;
   t.live += __popc(m);
-  c.map_writes += __popc(m);
+  count_writes(c, __popc(m));
   t_publish(c, t);
+  return true;
+}
+// t_claim_ok for a scratch table (never grows, no descriptor to publish to).
+__device__ __forceinline__ bool s_claim_ok(Ctx& c, Table& t, bool pred, uint32_t& slot) {
+  const uint32_t m = __ballot_sync(FULL, pred);
+  const uint32_t n = t.n, nn = n + __popc(m);
+  slot = n + __popc(m & lanemask_lt());
+  if (nn > t.cap) {
+    fail_cap(c, CAP_TABLE, t.cap);
+    return false;
+  }
+  t.n = nn;
+  t.live += __popc(m);
+  count_writes(c, __popc(m));
   return true;
 }
 // Claims k consecutive slots per lane; returns this lane's first slot.
@@ -497,7 +507,7 @@ __device__ __forceinline__ uint32_t t_claim_n(Ctx& c, Table& t, uint32_t k) {
   if (t.n + total > t.cap && !t_grow(c, t, t.n + total)) return NONE;
   t.n += total;
   t.live += total;
-  c.map_writes += total;
+  count_writes(c, total);
   t_publish(c, t);
   return first;
 }
@@ -638,7 +648,7 @@ __device__ void t_query(Ctx& c, const Table& src, uint32_t key, const Bx& q, Tab
   DT_START(dt);
   Table out = out_ref;  // header in registers while scanning
   const uint32_t n = src.n;
-  c.map_reads += n;
+  count_reads(c, n);
   for (uint32_t base = 0; base < n; base += 32) {
     const uint32_t i = base + laneid();
     bool hit = false;
@@ -658,7 +668,7 @@ __device__ void t_query(Ctx& c, const Table& src, uint32_t key, const Bx& q, Tab
     }
     if (!__any_sync(FULL, hit)) continue;
     uint32_t s;
-    if (!t_claim_ok(c, out, hit, s)) break;
+    if (!s_claim_ok(c, out, hit, s)) break;
     if (hit) t_put(out, s, 0, is, v0, v1, v2);
   }
   __syncwarp();
@@ -758,45 +768,49 @@ __device__ __forceinline__ void t_set(Ctx& c, Table& t_ref, uint32_t key, const 
   t_ref = t;
 }
 
+// Merges entry i into an entry with equal key and values whose union with it
+// is a box, the result into another such one, and so on.
+__device__ __forceinline__ void t_merge_entry(Ctx& c, Table& t, uint32_t i) {
+  uint32_t cand = i;
+  for (int guard = 0; guard < 4096; ++guard) {
+    DT_COUNT(N_MERGE_PROBE, 1);
+    const Ent ce = t_ent(t, cand);
+    const uint32_t k = ce.key;
+    if (k == DEAD) break;
+    const Bx e = ce.b;
+    const uint32_t v0 = ce.v0, v1 = ce.v1, v2 = ce.v2;
+    Bx jb{};
+    const uint32_t j = warp_find_first(c, t.n, [&](uint32_t x) {
+      const Ent f = t_ent(t, x);
+      const bool m = x != cand && f.key == k && f.v0 == v0 && f.v1 == v1 && f.v2 == v2 && bx_mergeable(e, f.b);
+      if (m) jb = f.b;
+      return m;
+    });
+    if (j == NONE) break;
+    const uint32_t src_lane = (j & 31u);
+    Bx jbb;
+    for (int d = 0; d < 3; ++d) {
+      jbb.lo[d] = __shfl_sync(FULL, jb.lo[d], src_lane);
+      jbb.hi[d] = __shfl_sync(FULL, jb.hi[d], src_lane);
+    }
+    const Bx u = bx_union(e, jbb);
+    __syncwarp();
+    if (laneid() == 0) {
+      t_put(t, j, k, u, v0, v1, v2);
+      t_kill(t, cand);
+    }
+    t_dead(c, t, 1);
+    __syncwarp();
+    cand = j;
+  }
+}
+
 // Merges entries from index `from` on with equal key and values into
 // adjacent entries whose union is a box (keeps the tables small).
 __device__ __noinline__ Table t_merge_from_v(Ctx& c, Table t, uint32_t from) {
   DT_START(dt);
   DT_COUNT(N_MERGE, 1);
-  for (uint32_t i = from; i < t.n; ++i) {
-    uint32_t cand = i;
-    for (int guard = 0; guard < 4096; ++guard) {
-      DT_COUNT(N_MERGE_PROBE, 1);
-      const Ent ce = t_ent(t, cand);
-      const uint32_t k = ce.key;
-      if (k == DEAD) break;
-      const Bx e = ce.b;
-      const uint32_t v0 = ce.v0, v1 = ce.v1, v2 = ce.v2;
-      Bx jb{};
-      const uint32_t j = warp_find_first(c, t.n, [&](uint32_t x) {
-        const Ent f = t_ent(t, x);
-        const bool m = x != cand && f.key == k && f.v0 == v0 && f.v1 == v1 && f.v2 == v2 && bx_mergeable(e, f.b);
-        if (m) jb = f.b;
-        return m;
-      });
-      if (j == NONE) break;
-      const uint32_t src_lane = (j & 31u);
-      Bx jbb;
-      for (int d = 0; d < 3; ++d) {
-        jbb.lo[d] = __shfl_sync(FULL, jb.lo[d], src_lane);
-        jbb.hi[d] = __shfl_sync(FULL, jb.hi[d], src_lane);
-      }
-      const Bx u = bx_union(e, jbb);
-      __syncwarp();
-      if (laneid() == 0) {
-        t_put(t, j, k, u, v0, v1, v2);
-        t_kill(t, cand);
-      }
-      t_dead(c, t, 1);
-      __syncwarp();
-      cand = j;
-    }
-  }
+  for (uint32_t i = from; i < t.n; ++i) t_merge_entry(c, t, i);
   DT_LAP(dt, D_MERGE);
   return t;
 }
@@ -877,7 +891,7 @@ __device__ uint32_t canonical(Ctx& c, const Table& in, uint32_t from, uint32_t t
     const Ent e = t_ent(in, from);
     if (e.key == DEAD || bx_empty(e.b)) return 0;
     uint32_t s;
-    if (!t_claim_ok(c, out, laneid() == 0, s)) return 0;
+    if (!s_claim_ok(c, out, laneid() == 0, s)) return 0;
     if (laneid() == 0) t_put(out, s, 0, e.b, 0, 0, 0);
     __syncwarp();
     pt_lap(pt, c, PH_CANON);
@@ -898,8 +912,8 @@ __device__ __noinline__ uint32_t canonical_impl(Ctx& c, const Table& in, uint32_
       b = t_box(in, i);
       live = !bx_empty(b);
     }
-    const uint32_t s = t_claim(c, W, live);
-    if (c.err) return 0;
+    uint32_t s;
+    if (!s_claim_ok(c, W, live, s)) return 0;
     if (live) t_put(W, s, 0, b, 0, 0, 0);
   }
   __syncwarp();
@@ -1169,15 +1183,29 @@ __device__ uint32_t find_alloc(Ctx& c, uint32_t buf, uint32_t mem, const Bx& b) 
   return k == NONE ? NONE : L[k];
 }
 
-// Per-lane variant (no warp collectives).
-__device__ bool covered_by_alloc(const Ctx& c, uint32_t buf, uint32_t mem, const Bx& b) {
+// Per-lane variant (no warp collectives): four allocations' records in
+// flight at a time, where a chain of dependent loads per allocation bounded
+// the lookups.
+__device__ __forceinline__ uint32_t lane_find_alloc(const Ctx& c, uint32_t buf, uint32_t mem, const Bx& b) {
+  static_assert(sizeof(AllocRec) == 48, "an allocation record is three 16-byte words");
   const AllocRec* A = c.nd->allocs;
   const uint32_t* L = c.nd->live;
-  for (uint32_t i = 0; i < c.n_live; ++i) {
-    const AllocRec& a = A[L[i]];
-    if (a.buffer == buf && a.mem == mem && bx_contains(alloc_box(a), b)) return true;
+  const uint32_t n = c.n_live;
+  for (uint32_t i = 0; i < n; i += 4) {
+    uint32_t id[4];
+    uint4 h[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) id[u] = L[i + u < n ? i + u : i];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) h[u] = *reinterpret_cast<const uint4*>(A + id[u]);  // buffer, mem, live, user
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u)
+      if (i + u < n && h[u].x == buf && h[u].y == mem && bx_contains(alloc_box(A[id[u]]), b)) return id[u];
   }
-  return false;
+  return NONE;
+}
+__device__ bool covered_by_alloc(const Ctx& c, uint32_t buf, uint32_t mem, const Bx& b) {
+  return lane_find_alloc(c, buf, mem, b) != NONE;
 }
 
 __device__ __forceinline__ const igs_task& task_of(const Ctx& c, uint32_t item) {
@@ -1224,23 +1252,33 @@ __device__ __noinline__ void task_chunks(Ctx& c, const igs_task& t, Table& CH) {
         b.hi[2] = t.range[2];
         ok = b.lo[0] < b.hi[0] && b.lo[1] < b.hi[1];
       }
-      const uint32_t s = t_claim(c, CH, ok);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, CH, ok, s)) return;
       if (ok) t_put(CH, s, i, b, node, mem, 0);
     }
     __syncwarp();
     return;
   }
   const uint64_t E0 = t.range[0], C = t.num_chunks, M = (uint64_t)c.N * c.D;
+  const bool narrow = (C + 1) * E0 <= 0xFFFFFFFFull && C * M <= 0xFFFFFFFFull;  // 32-bit divisions do
   for (uint32_t base = 0; base < t.num_chunks; base += 32) {
     const uint32_t i = base + laneid();
     bool ok = false;
     Bx b{};
     uint32_t node = 0, mem = 0;
     if (i < t.num_chunks) {
-      const uint32_t r0 = (uint32_t)((uint64_t)i * E0 / C), r1 = (uint32_t)((uint64_t)(i + 1) * E0 / C);
+      uint32_t r0, r1, g;
+      if (narrow) {
+        const uint32_t e0 = (uint32_t)E0, nc = (uint32_t)C;
+        r0 = i * e0 / nc;
+        r1 = (i + 1) * e0 / nc;
+        g = i * (uint32_t)M / nc;
+      } else {
+        r0 = (uint32_t)((uint64_t)i * E0 / C);
+        r1 = (uint32_t)((uint64_t)(i + 1) * E0 / C);
+        g = (uint32_t)((uint64_t)i * M / C);
+      }
       ok = r0 < r1;
-      const uint32_t g = (uint32_t)((uint64_t)i * M / C);
       node = g / c.D;
       mem = 2 + g % c.D;
       b.lo[0] = r0;
@@ -1250,8 +1288,8 @@ __device__ __noinline__ void task_chunks(Ctx& c, const igs_task& t, Table& CH) {
         b.hi[d] = t.range[d];
       }
     }
-    const uint32_t s = t_claim(c, CH, ok);
-    if (c.err) return;
+    uint32_t s;
+    if (!s_claim_ok(c, CH, ok, s)) return;
     if (ok) t_put(CH, s, i, b, node, mem, 0);
   }
   __syncwarp();
@@ -1387,7 +1425,7 @@ __device__ __forceinline__ bool emit_deps(Ctx& c, const Acc* acc, int nacc, bool
       const uint32_t n = snap ? c.snap_n[tab] : dsc[2];
       if (n == 0) continue;
       const uint32_t* tb = snap ? c.snap_tab[tab] : nd->heap + (size_t)dsc[0] * F_COUNT;
-      c.map_reads += n;
+      count_reads(c, n);
       DT_COUNT(N_PROBE_ENTRIES, n);
       for (uint32_t base = 0; base < n; base += 32) {
         const uint32_t f = base + laneid();
@@ -1418,7 +1456,7 @@ __device__ __forceinline__ bool emit_deps(Ctx& c, const Acc* acc, int nacc, bool
         }
         if (!__any_sync(FULL, hit)) continue;
         uint32_t s;
-        if (!t_claim_ok(c, D, hit, s)) {
+        if (!s_claim_ok(c, D, hit, s)) {
           c.s[S_DEP] = D;
           return false;
         }
@@ -1445,16 +1483,31 @@ __device__ __forceinline__ bool emit_deps(Ctx& c, const Acc* acc, int nacc, bool
 // The unique predecessors in S_DEP, ascending, kinds OR-ed, as edges into
 // instruction id, written to out[0, count) (at most cap of them, else a
 // capacity failure of kind cap_kind); marks each predecessor as having a
-// successor. Returns the count (NONE on failure).
+// successor. Returns the count (NONE on failure). sorted: S_DEP holds unique
+// predecessors in ascending order, none of them staged.
 __device__ __forceinline__ uint32_t emit_edges(Ctx& c, uint32_t id, igs_edge* out, uint32_t cap, CapKind cap_kind,
-                                            uint32_t cap_report) {
+                                            uint32_t cap_report, bool sorted = false) {
   if (c.err) return NONE;
   NodeDev* nd = c.nd;
   const Table& D = c.s[S_DEP];
   // unique predecessors in ascending order, kinds OR-ed
   const uint32_t nd0 = D.n;
   uint32_t n_unique = 0;
-  if (nd0 <= 32) {
+  if (sorted) {
+    if (nd0 > cap) {
+      fail_cap(c, cap_kind, cap_report);
+      return NONE;
+    }
+    for (uint32_t i = laneid(); i < nd0; i += 32) {
+      igs_edge e;
+      e.from = FLD(D, F_V, i);
+      e.to = id;
+      e.kind = FLD(D, F_V + 1, i);
+      out[i] = e;
+      nd->has_succ[e.from] = 1;
+    }
+    n_unique = nd0;
+  } else if (nd0 <= 32) {
     // one entry per lane: the first lane of each group of equal predecessors
     // leads it; a leader's kind ORs its group's kinds and its rank counts the
     // leaders with smaller ids (one pass over the groups)
@@ -1621,9 +1674,12 @@ __device__ __forceinline__ bool apply_read(Ctx& c, uint32_t aid, uint32_t n, G b
   for (uint32_t r = 0; r < n; ++r) {
     Bx q;
     if (!box(r, q)) continue;
-    if (again) t_subtract(c, RD, NONE, q, id);
-    const uint32_t s = t_claim(c, RD, laneid() == 0);
-    if (c.err) return false;
+    if (again) {
+      t_subtract(c, RD, NONE, q, id);
+      if (c.err) return false;
+    }
+    uint32_t s;
+    if (!t_claim_ok(c, RD, laneid() == 0, s)) return false;
     if (laneid() == 0) t_put(RD, s, 0, q, id, 0, 0);
     __syncwarp();
   }
@@ -1749,7 +1805,12 @@ __device__ __noinline__ uint32_t emit_impl(Ctx& c, uint32_t type, uint32_t seq, 
   DT_COUNT(N_EMIT, 1);
   if (!emit_deps(c, acc, nacc, keep_dep)) return NONE;
   DT_LAP(dt, D_PROBE);
-  const uint32_t ne = emit_edges(c, id, nd->edges + c.n_edge, nd->cap_edge - c.n_edge, CAP_EDGE, nd->cap_edge);
+  // a horizon's or epoch's predecessors were collected by ascending id, each
+  // once (some hundred after a few tasks: comparing them all took 36 us a
+  // task of N-body on 8 x 4 devices)
+  const bool front = (type == IGS_HORIZON || type == IGS_EPOCH) && nacc == 0;
+  const uint32_t ne =
+      emit_edges(c, id, nd->edges + c.n_edge, nd->cap_edge - c.n_edge, CAP_EDGE, nd->cap_edge, front);
   if (ne == NONE) return NONE;
   c.n_edge += ne;
   DT_LAP(dt, D_DEDUP);
@@ -1839,8 +1900,8 @@ __device__ __noinline__ void emit_free(Ctx& c, uint32_t seq, uint32_t aid) {
     for (uint32_t base = 0; base < T.n; base += 32) {
       const uint32_t i = base + laneid();
       const bool hit = i < T.n && t_key(T, i) != DEAD;
-      const uint32_t s = t_claim(c, D, hit);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, D, hit, s)) return;
       if (hit) {
         FLD(D, F_V, s) = t_v(T, 0, i);
         FLD(D, F_V + 1, s) = IGS_DEP_ALLOC;
@@ -1928,8 +1989,8 @@ __device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_
     for (uint32_t base = 0; base < Q.n; base += 32) {
       const uint32_t i = base + laneid();
       const bool hit = i < Q.n && t_v(Q, 0, i) == prod && t_v(Q, 1, i) == pmem;
-      const uint32_t s = t_claim(c, G, hit);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, G, hit, s)) return;
       if (hit) t_put(G, s, 0, t_box(Q, i), 0, 0, 0);
     }
     __syncwarp();
@@ -1946,8 +2007,8 @@ __device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_
           is = bx_isect(t_box(G, i), ab);
           hit = !bx_empty(is);
         }
-        const uint32_t s = t_claim(c, P, hit);
-        if (c.err) return false;
+        uint32_t s;
+        if (!s_claim_ok(c, P, hit, s)) return false;
         if (hit) t_put(P, s, 0, is, 0, 0, 0);
       }
       __syncwarp();
@@ -1976,8 +2037,8 @@ __device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_
           return false;
         }
         t_reset(P);  // P now holds the allocation's box
-        const uint32_t s0 = t_claim(c, P, laneid() == 0);
-        if (c.err) return false;
+        uint32_t s0;
+        if (!s_claim_ok(c, P, laneid() == 0, s0)) return false;
         if (laneid() == 0) t_put(P, s0, 0, bb, 0, 0, 0);
         __syncwarp();
         const uint32_t hid = c.n_alloc;
@@ -1987,8 +2048,8 @@ __device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_
         c.n_alloc += 1;
         {
           Table WR = wr_t(c, hid);
-          const uint32_t s1 = t_claim(c, WR, laneid() == 0);
-          if (c.err) return false;
+          uint32_t s1;
+          if (!t_claim_ok(c, WR, laneid() == 0, s1)) return false;
           if (laneid() == 0) t_put(WR, s1, 0, bb, iid, 1, 0);  // v1 = 1: the writer is an allocation
           __syncwarp();
         }
@@ -2009,8 +2070,8 @@ __device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_
       for (uint32_t base = 0; base < (plan ? 0u : CN.n); base += 32) {
         const uint32_t i = base + laneid();
         const bool in = i < CN.n;
-        const uint32_t s = t_claim(c, CP, in);
-        if (c.err) return false;
+        uint32_t s;
+        if (!s_claim_ok(c, CP, in, s)) return false;
         if (in) t_put(CP, s, 0, t_box(CN, i), 0, 0, 0);
       }
       __syncwarp();
@@ -2245,8 +2306,8 @@ __device__ __noinline__ void a3_buffer(Ctx& c, const igs_task& t, uint32_t seq, 
     for (uint32_t base = 0; base < TMP.n; base += 32) {
       const uint32_t i = base + laneid();
       const bool live = i < TMP.n && t_key(TMP, i) != DEAD;
-      const uint32_t s = t_claim(c, MISS, live);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, MISS, live, s)) return;
       if (live) t_put(MISS, s, 0, t_box(TMP, i), m, 0, 0);
     }
     __syncwarp();
@@ -2258,8 +2319,8 @@ __device__ __noinline__ void a3_buffer(Ctx& c, const igs_task& t, uint32_t seq, 
     for (uint32_t base = 0; base < MISS.n; base += 32) {
       const uint32_t i = base + laneid();
       const bool hit = i < MISS.n && t_v(MISS, 0, i) == c.node;
-      const uint32_t s = t_claim(c, sel, hit);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, sel, hit, s)) return;
       if (hit) t_put(sel, s, 0, t_box(MISS, i), 0, 0, 0);
     }
     __syncwarp();
@@ -2271,8 +2332,8 @@ __device__ __noinline__ void a3_buffer(Ctx& c, const igs_task& t, uint32_t seq, 
       for (uint32_t base = 0; base < CN.n + 1; base += 32) {
         const uint32_t i = base + laneid();
         const bool in = i < CN.n + 1;
-        const uint32_t s = t_claim(c, OUT, in);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, OUT, in, s)) return;
         if (in) {
           if (i < CN.n) t_put(OUT, s, seq, t_box(CN, i), 1, b, NONE);
           else t_put(OUT, s, seq, bb, 3, b, NONE);
@@ -2299,8 +2360,8 @@ __device__ __noinline__ void a3_buffer(Ctx& c, const igs_task& t, uint32_t seq, 
     for (uint32_t base = 0; base < CN.n + 1; base += 32) {
       const uint32_t i = base + laneid();
       const bool in = i < CN.n + 1;
-      const uint32_t s = t_claim(c, OUT, in);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, OUT, in, s)) return;
       if (in) {
         if (i < CN.n) t_put(OUT, s, seq, t_box(CN, i), 0, b, m);
         else t_put(OUT, s, seq, bb, 2, b, m);
@@ -2438,8 +2499,8 @@ __device__ __noinline__ void requirements(Ctx& c, const igs_task& t, uint32_t se
         hit = !bx_empty(x) && (only_key == NONE || key == only_key);
       }
     }
-    const uint32_t s = t_claim(c, RQ, hit);
-    if (c.err) return;
+    uint32_t s;
+    if (!s_claim_ok(c, RQ, hit, s)) return;
     if (hit) t_put(RQ, s, key, x, own_flag, 0, 0);
   }
   uint32_t qs, qe;
@@ -2453,8 +2514,8 @@ __device__ __noinline__ void requirements(Ctx& c, const igs_task& t, uint32_t se
       key = t_v(c.qr, 1, i) * 32 + 1;
       hit = (kind == 2 || kind == 3) && (only_key == NONE || key == only_key);
     }
-    const uint32_t s = t_claim(c, RQ, hit);
-    if (c.err) return;
+    uint32_t s;
+    if (!s_claim_ok(c, RQ, hit, s)) return;
     if (hit) t_put(RQ, s, key, t_box(c.qr, i), own_flag, 0, 0);
   }
   __syncwarp();
@@ -2487,6 +2548,27 @@ __device__ __noinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq
   t_reset(RQ);
   requirements(c, t, seq, CH, MP, RQ, NONE, 1);
   if (c.err) return;
+  // only those outside every allocation matter, and a (buffer, memory) pair's
+  // allocations change below only when its turn comes: looked up once
+  uint32_t n_need = 0;
+  for (uint32_t base = 0; base < RQ.n; base += 32) {
+    const uint32_t i = base + laneid();
+    bool need = false;
+    uint32_t key = 0;
+    Bx x{};
+    if (i < RQ.n) {
+      const Ent e = t_ent(RQ, i);
+      key = e.key;
+      x = e.b;
+      need = !covered_by_alloc(c, key >> 5, key & 31u, x);
+    }
+    __syncwarp();
+    const uint32_t m = __ballot_sync(FULL, need);
+    if (need) t_put(RQ, n_need + __popc(m & lanemask_lt()), key, x, 1, 0, 0);
+    n_need += __popc(m);
+    __syncwarp();
+  }
+  RQ.n = RQ.live = n_need;
   // the requirements of every task still queued (lookahead, Sec. 4.3), found
   // once for all (buffer, memory) pairs where they fit the table; else they
   // are found again for each pair
@@ -2534,10 +2616,10 @@ __device__ __noinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq
       Bx x{};
       if (i < RQ.n && t_key(RQ, i) == key) {
         x = t_box(RQ, i);
-        hit = !covered_by_alloc(c, b, m, x);
+        hit = true;
       }
-      const uint32_t s = t_claim(c, CL, hit);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, CL, hit, s)) return;
       if (hit) t_put(CL, s, 0, x, 1, 0, 0);
     }
     __syncwarp();
@@ -2552,8 +2634,8 @@ __device__ __noinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq
         hit = !covered_by_alloc(c, b, m, x);
       }
       if (!__any_sync(FULL, hit)) continue;
-      const uint32_t s = t_claim(c, CL, hit);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, CL, hit, s)) return;
       if (hit) t_put(CL, s, 0, x, 0, 0, 0);
     }
     __syncwarp();
@@ -2703,8 +2785,8 @@ __device__ __noinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq
       c.n_alloc += 1;
       {
         Table WR = wr_t(c, aid);
-        const uint32_t s = t_claim(c, WR, laneid() == 0);
-        if (c.err) return;
+        uint32_t s;
+        if (!t_claim_ok(c, WR, laneid() == 0, s)) return;
         if (laneid() == 0) t_put(WR, s, 0, bb, iid, 1, 0);  // v1 = 1: the writer is an allocation
         __syncwarp();
       }
@@ -2714,8 +2796,8 @@ __device__ __noinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq
       for (uint32_t base = 0; base < c.n_live; base += 32) {
         const uint32_t x = base + laneid();
         const bool hit = x < c.n_live && L[x] != aid && A[L[x]].mark == ci;
-        const uint32_t s = t_claim(c, AB, hit);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, AB, hit, s)) return;
         if (hit) FLD(AB, F_V, s) = L[x];
       }
       __syncwarp();
@@ -2836,8 +2918,8 @@ __device__ bool p4_consumer(Ctx& c, const igs_task& t, uint32_t seq, const Table
   }
   Table& RG = c.s[S_RG];
   t_reset(RG);
-  const uint32_t s = t_claim(c, RG, laneid() == 0);
-  if (c.err) return false;
+  uint32_t s;
+  if (!s_claim_ok(c, RG, laneid() == 0, s)) return false;
   if (laneid() == 0) t_put(RG, s, 0, x, 0, 0, 0);
   __syncwarp();
   coherence(c, seq, b, mem, dst, RG, 0, 1);
@@ -3289,16 +3371,16 @@ __device__ __noinline__ void p5_state(Ctx& c, const igs_task& t, const Table& CH
           kid = FLD(AL, F_V, slot * na);
           mem = t_v(CH, 1, slot);
         }
-        const uint32_t s = t_claim(c, B, hit);
-        if (c.err) return;
+        uint32_t s;
+        if (!t_claim_ok(c, B, hit, s)) return;
         if (hit) t_put(B, s, 0, x, kid, mem, 1u << mem);
       }
       for (uint32_t m = 0; m < c.N; ++m) {
         if (m == c.node || t_key(NB, m) == DEAD) continue;
         const Bx x = map_box(t.acc[a], t_box(NB, m), bd);
         if (bx_empty(x)) continue;
-        const uint32_t s = t_claim(c, B, laneid() == 0);
-        if (c.err) return;
+        uint32_t s;
+        if (!t_claim_ok(c, B, laneid() == 0, s)) return;
         if (laneid() == 0) t_put(B, s, 0, x, REMOTE, 0, 0);
         __syncwarp();
       }
@@ -3613,8 +3695,8 @@ __device__ __noinline__ void p2_pushes(Ctx& c, uint32_t seq, uint32_t qs, uint32
     for (uint32_t base = g0; base < g1; base += 32) {
       const uint32_t i = base + laneid();
       const bool in = i < g1;
-      const uint32_t s = t_claim(c, RG, in);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, RG, in, s)) return;
       if (in) t_put(RG, s, 0, t_box(c.qr, i), 0, 0, 0);
     }
     __syncwarp();
@@ -3650,8 +3732,8 @@ __device__ __noinline__ void p2_pushes(Ctx& c, uint32_t seq, uint32_t qs, uint32
       for (uint32_t base = 0; base < Q.n; base += 32) {
         const uint32_t i = base + laneid();
         const bool hit = i < Q.n && (((uint64_t)t_v(Q, 0, i) << 32) | t_v(Q, 1, i)) == best;
-        const uint32_t s = t_claim(c, G, hit);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, G, hit, s)) return;
         if (hit) t_put(G, s, 0, t_box(Q, i), 0, 0, 0);
       }
       __syncwarp();
@@ -3688,8 +3770,8 @@ __device__ __noinline__ void p3_group(Ctx& c, const igs_task& t, uint32_t seq, c
   for (uint32_t base = g0; base < g1; base += 32) {
     const uint32_t i = base + laneid();
     const bool in = i < g1;
-    const uint32_t s = t_claim(c, RG, in);
-    if (c.err) return;
+    uint32_t s;
+    if (!s_claim_ok(c, RG, in, s)) return;
     if (in) t_put(RG, s, 0, t_box(qr, i), 0, 0, 0);
   }
   __syncwarp();
@@ -3722,8 +3804,8 @@ __device__ __noinline__ void p3_group(Ctx& c, const igs_task& t, uint32_t seq, c
           is = bx_isect(t_box(RG, i), x);
           hit = !bx_empty(is);
         }
-        const uint32_t s = t_claim(c, CONS, hit);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, CONS, hit, s)) return;
         if (hit) t_put(CONS, s, 0, is, ncons, 0, 0);
       }
       __syncwarp();
@@ -3757,8 +3839,8 @@ __device__ __noinline__ void p3_group(Ctx& c, const igs_task& t, uint32_t seq, c
       for (uint32_t base = 0; base < CONS.n; base += 32) {
         const uint32_t i = base + laneid();
         const bool hit = i < CONS.n && t_v(CONS, 0, i) == k;
-        const uint32_t s = t_claim(c, G, hit);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, G, hit, s)) return;
         if (hit) t_put(G, s, 0, t_box(CONS, i), 0, 0, 0);
       }
       __syncwarp();
@@ -3798,8 +3880,8 @@ __device__ __noinline__ void p3_group(Ctx& c, const igs_task& t, uint32_t seq, c
       for (uint32_t base = 0; base < CN.n; base += 32) {
         const uint32_t i = base + laneid();
         const bool in = i < CN.n;
-        const uint32_t s = t_claim(c, COV, in);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, COV, in, s)) return;
         if (in) t_put(COV, s, 0, t_box(CN, i), 0, 0, 0);
       }
       __syncwarp();
@@ -4073,17 +4155,22 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
           if (hit) {
             const uint32_t b = t.acc[a].buffer, m = t_v(CH, 1, slot);
             const Table B = heap_table(c.nd, c.nd->bst_d + kDesc * b);
-            for (uint32_t j = 0; j < B.n; ++j) {
-              if (t_key(B, j) == DEAD || !bx_overlap(t_box(B, j), x)) continue;
-              const uint32_t prod = t_v(B, 0, j), mask = t_v(B, 2, j);
-              if (prod == NONE) flags |= 1u;
-              else if (!((mask >> m) & 1u)) flags |= 2u;
+            for (uint32_t j = 0; j < B.n; j += 4) {  // four entries' loads in flight
+              Ent e[4];
+#pragma unroll
+              for (uint32_t u = 0; u < 4; ++u) e[u] = t_ent(B, j + u < B.n ? j + u : j);
+#pragma unroll
+              for (uint32_t u = 0; u < 4; ++u) {
+                if (e[u].key == DEAD || !bx_overlap(e[u].b, x)) continue;
+                if (e[u].v0 == NONE) flags |= 1u;
+                else if (!((e[u].v2 >> m) & 1u)) flags |= 2u;
+              }
             }
           }
         }
       }
-      const uint32_t s = t_claim(c, PC, hit);
-      if (c.err) return;
+      uint32_t s;
+      if (!s_claim_ok(c, PC, hit, s)) return;
       if (hit) t_put(PC, s, flags, x, i, 0, 0);
     }
     __syncwarp();
@@ -4147,8 +4234,6 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
       fail_cap(c, CAP_TABLE, AL.cap);
       return;
     }
-    const AllocRec* A = c.nd->allocs;
-    const uint32_t* L = c.nd->live;
     for (uint32_t base = 0; base < total; base += 32) {
       const uint32_t i = base + laneid();
       if (i < total) {
@@ -4157,11 +4242,7 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
         if (t_v(CH, 0, slot) == c.node) {
           const Bx x = t_box(MP, i);
           if (!bx_empty(x)) {
-            const uint32_t buf = t.acc[a].buffer, mem = t_v(CH, 1, slot);
-            for (uint32_t k = 0; k < c.n_live && al == NONE; ++k) {
-              const AllocRec& r = A[L[k]];
-              if (r.buffer == buf && r.mem == mem && bx_contains(alloc_box(r), x)) al = L[k];
-            }
+            al = lane_find_alloc(c, t.acc[a].buffer, t_v(CH, 1, slot), x);
             if (al == NONE) al = NONE - 1;  // missing: an internal error
           }
         }
@@ -4228,15 +4309,15 @@ __device__ __noinline__ void process(Ctx& c, uint32_t item) {
         if (!new_alloc(c, aid, it.arg, 0, dom, 1)) return;
         c.n_alloc += 1;
         Table WR = wr_t(c, aid);
-        const uint32_t s = t_claim(c, WR, laneid() == 0);
-        if (c.err) return;
+        uint32_t s;
+        if (!t_claim_ok(c, WR, laneid() == 0, s)) return;
         if (laneid() == 0) t_put(WR, s, 0, dom, c.epoch, 0, 0);
-        const uint32_t s2 = t_claim(c, B, laneid() == 0);
-        if (c.err) return;
+        uint32_t s2;
+        if (!t_claim_ok(c, B, laneid() == 0, s2)) return;
         if (laneid() == 0) t_put(B, s2, 0, dom, c.epoch, 0, 1u);
       } else {
-        const uint32_t s2 = t_claim(c, B, laneid() == 0);
-        if (c.err) return;
+        uint32_t s2;
+        if (!t_claim_ok(c, B, laneid() == 0, s2)) return;
         if (laneid() == 0) t_put(B, s2, 0, dom, NONE, 0, 0);
       }
       __syncwarp();
@@ -4252,8 +4333,8 @@ __device__ __noinline__ void process(Ctx& c, uint32_t item) {
       for (uint32_t base = c.last_sync; base < c.n_instr; base += 32) {
         const uint32_t i = base + laneid();
         const bool f = i < c.n_instr && !c.nd->has_succ[i];
-        const uint32_t s = t_claim(c, D, f);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, D, f, s)) return;
         if (f) {
           FLD(D, F_V, s) = i;
           FLD(D, F_V + 1, s) = IGS_DEP_FRONT;
@@ -4283,8 +4364,8 @@ __device__ __noinline__ void process(Ctx& c, uint32_t item) {
       for (uint32_t base = 0; base < c.n_live; base += 32) {
         const uint32_t x = base + laneid();
         const bool hit = x < c.n_live && c.nd->allocs[c.nd->live[x]].buffer == b;
-        const uint32_t s = t_claim(c, AB, hit);
-        if (c.err) return;
+        uint32_t s;
+        if (!s_claim_ok(c, AB, hit, s)) return;
         if (hit) FLD(AB, F_V, s) = c.nd->live[x];
       }
       __syncwarp();
@@ -4380,8 +4461,8 @@ __device__ __noinline__ void record_queued_reqs(Ctx& c, const igs_task& t, uint3
   for (uint32_t base = 0; base < RQ.n && !c.err; base += 32) {
     const uint32_t i = base + laneid();
     const bool in = i < RQ.n;
-    const uint32_t s = t_claim(c, c.qr, in);
-    if (c.err) return;
+    uint32_t s;
+    if (!s_claim_ok(c, c.qr, in, s)) return;
     if (in) t_put(c.qr, s, seq, t_box(RQ, i), QR_QUEUED_REQ, t_key(RQ, i), 0);
   }
   __syncwarp();
@@ -4400,8 +4481,8 @@ __device__ void own_create(Ctx& c, const Item& it) {
   const BufDesc& bd = buf_of(c, it.arg);
   if (!table_new(c, c.nd->own_d + kDesc * it.arg, 32)) return;
   Table O = own_t(c, it.arg);
-  const uint32_t s = t_claim(c, O, laneid() == 0);
-  if (c.err) return;
+  uint32_t s;
+  if (!t_claim_ok(c, O, laneid() == 0, s)) return;
   if (laneid() == 0) t_put(O, s, 0, buffer_box(bd), bd.init ? HOST : NONE, 0xFFFFFFFFu, 0);
   __syncwarp();
 }
