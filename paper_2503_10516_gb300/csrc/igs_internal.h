@@ -234,6 +234,9 @@ size_t igs_lower_pool_words(uint32_t cap_scratch, uint32_t front_cap);
 int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                           uint32_t blocks, uint32_t* scratch_dev, uint32_t cap_scratch, uint32_t front_cap,
                           void* stream);
+// What every node's state starts with: initial epoch, empty tables, all
+// allocation slots free.
+int igs_launch_init_nodes(const igs::NodeDev* nodes_dev, uint32_t n, void* stream);
 // One block per unit.
 // reserve: each unit's block also holds most of its SM's registers, keeping
 // other kernels off the SMs that lower (used while the executor runs concurrently).

@@ -4994,6 +4994,19 @@ __device__ __noinline__ void stage_submissions(const ProgDev* pg, uint32_t from,
   __syncwarp();
 }
 
+// What a node's state starts with: block n resets node n.
+__global__ void init_nodes_kernel(const NodeDev* nodes) {
+  const NodeDev& nd = nodes[blockIdx.x];
+  const uint32_t desc = kDesc * (2 * nd.cap_buffers + 2 * nd.cap_slots);
+  for (uint32_t i = threadIdx.x; i < desc; i += blockDim.x) nd.own_d[i] = 0;
+  for (uint32_t i = threadIdx.x; i < nd.cap_slots; i += blockDim.x)
+    nd.free_slots[i] = nd.cap_slots - 1 - i;  // pops 0, 1, 2, ...
+  if (threadIdx.x == 0) {
+    nd.has_succ[0] = 0;
+    nd.instrs[0] = igs_instruction{0, IGS_EPOCH, NONE, NONE, NONE, NONE, NONE, 0, 0, 0, 0};
+  }
+}
+
 // Serving loop: warp w serves slot w; it takes every submission published so
 // far, then publishes its progress. Waits are bounded: after idle_polls empty
 // polls (about 2 us each) the warp leaves with EXIT_IDLE; a set stop flag ends
@@ -5069,6 +5082,11 @@ __global__ void __launch_bounds__(32) serve_kernel(ServeSlot* slots, uint32_t n_
 
 }  // namespace
 }  // namespace igs
+
+int igs_launch_init_nodes(const igs::NodeDev* nodes_dev, uint32_t n, void* stream) {
+  igs::init_nodes_kernel<<<n, 256, 0, (cudaStream_t)stream>>>(nodes_dev);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
 
 int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t* stop, uint64_t idle_polls, void* stream) {
   if (n_slots == 0) return 0;

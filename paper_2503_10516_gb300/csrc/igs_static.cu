@@ -68,20 +68,6 @@ Layout layout(uint32_t cap_instr) {
   return L;
 }
 
-// What a node's state starts with (the arrays keep the previous call's
-// contents): block n resets node n.
-__global__ void static_init(const igs::NodeDev* nodes) {
-  using namespace igs;
-  const NodeDev nd = nodes[blockIdx.x];
-  const uint32_t desc = kDesc * (2 * kBuffers + 2 * kSlots);
-  for (uint32_t i = threadIdx.x; i < desc; i += blockDim.x) nd.own_d[i] = 0;
-  for (uint32_t i = threadIdx.x; i < kSlots; i += blockDim.x) nd.free_slots[i] = kSlots - 1 - i;  // pops 0, 1, 2, ...
-  if (threadIdx.x == 0) {
-    nd.has_succ[0] = 0;
-    nd.instrs[0] = igs_instruction{0, IGS_EPOCH, NONE, NONE, NONE, NONE, NONE, 0, 0, 0, 0};
-  }
-}
-
 // Counts and status of every node into the caller's words, and what the host
 // reads back: {status, rejected tasks} per node.
 struct CountPtrs {
@@ -307,7 +293,7 @@ extern "C" int igs_lower_static(const igs_config* cfg, const igs_static_buffer* 
     for (uint32_t n = 0; n < N; ++n)
       nodes[n].helper_scratch = helped ? reinterpret_cast<uint32_t*>(helpers + kHelperBytes * n) : nullptr;
     CKS(cudaMemcpyAsync(base, stage.data(), o_state, cudaMemcpyHostToDevice, stream));
-    static_init<<<N, 128, 0, stream>>>(d_nodes);
+    if (igs_launch_init_nodes(d_nodes, N, stream)) return IGS_ERR_CUDA;
     if (igs_launch_lower(reinterpret_cast<const Unit*>(base + o_units), N, NONE, stream, false, nullptr, helped != 0))
       return IGS_ERR_CUDA;
     static_counts<<<1, 32, 0, stream>>>(d_nodes, N, counts, reinterpret_cast<uint32_t*>(base + o_result));
