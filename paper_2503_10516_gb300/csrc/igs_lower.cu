@@ -342,6 +342,7 @@ __device__ bool heap_lock(Ctx& c) {
   }
   ok = __shfl_sync(FULL, ok, 0);
   if (!ok) fail(c, ST_TIMEOUT);
+  __syncwarp();
   return ok != 0;
 }
 __device__ void heap_unlock(Ctx& c) {
@@ -359,17 +360,18 @@ __device__ __noinline__ uint32_t heap_alloc(Ctx& c, uint32_t entries, uint32_t& 
   cap = 32u << k;
   NodeDev* nd = c.nd;
   if (!heap_lock(c)) return NONE;
-  volatile uint32_t* fh = nd->free_head;
-  __syncwarp();
+  // plain loads: what other warps of the block wrote under the lock is ordered
+  // by it and in this SM's L1 (volatile ones went to L2, several in a row)
+  uint32_t* fh = nd->free_head;
   const uint32_t head = fh[k];
   if (head != NONE) {
-    const uint32_t next = reinterpret_cast<volatile uint32_t*>(nd->heap)[(size_t)head * F_COUNT];
+    const uint32_t next = nd->heap[(size_t)head * F_COUNT];
     __syncwarp();
     if (laneid() == 0) fh[k] = next;
     heap_unlock(c);
     return head;
   }
-  volatile uint32_t* vtop = &nd->heap_top;
+  uint32_t* vtop = &nd->heap_top;
   const uint32_t top = c.lock ? *vtop : c.heap_top;
   if ((uint64_t)top + cap > nd->cap_heap) {
     heap_unlock(c);
@@ -390,10 +392,10 @@ __device__ void heap_free(Ctx& c, uint32_t off, uint32_t cap) {
   const int k = heap_class(cap);
   NodeDev* nd = c.nd;
   if (!heap_lock(c)) return;
-  volatile uint32_t* fh = nd->free_head;
+  uint32_t* fh = nd->free_head;
   __syncwarp();
   if (laneid() == 0) {
-    reinterpret_cast<volatile uint32_t*>(nd->heap)[(size_t)off * F_COUNT] = fh[k];
+    nd->heap[(size_t)off * F_COUNT] = fh[k];
     fh[k] = off;
   }
   heap_unlock(c);
@@ -1151,10 +1153,16 @@ __device__ void drop_alloc(Ctx& c, uint32_t aid) {
   if (laneid() == 0) {
     c.nd->allocs[aid].live = 0;
     c.nd->free_slots[c.n_free] = slot;
-    uint32_t* L = c.nd->live;
-    uint32_t k = 0;
-    while (k < c.n_live && L[k] != aid) ++k;
-    for (; k + 1 < c.n_live; ++k) L[k] = L[k + 1];
+  }
+  // the live list closes up, 32 ids at a time
+  uint32_t* L = c.nd->live;
+  const uint32_t n = c.n_live, k = warp_find_first(c, n, [&](uint32_t i) { return L[i] == aid; });
+  for (uint32_t base = k; base < n; base += 32) {  // k is NONE (no pass) if it is not listed
+    const uint32_t i = base + laneid();
+    const uint32_t id = i + 1 < n ? L[i + 1] : 0u;
+    __syncwarp();
+    if (i + 1 < n) L[i] = id;
+    __syncwarp();
   }
   c.n_free += 1;
   c.n_live -= 1;
@@ -2928,7 +2936,7 @@ __device__ bool p4_consumer(Ctx& c, const igs_task& t, uint32_t seq, const Table
 
 // Coherence with several warps (Sec. 3.3, a5), in two shared phases.
 // Plan: worker p4_worker(b, m) takes, in consumer order, the stale consumers
-// of buffer b on memory m whose regions meet another one of that pair (the
+// of buffer b on memory m whose stale parts meet another one's of that pair (the
 // others go to the workers in turn) and stages their copies (records, boxes,
 // edges) without changing any table. Planning against the tables as they were
 // before the phase gives the single-warp path's copies and edges: a copy
@@ -3350,7 +3358,14 @@ __device__ __noinline__ void p5_state(Ctx& c, const igs_task& t, const Table& CH
     const BufDesc& bd = buf_of(c, t.acc[a].buffer);
     Table B = bst_t(c, t.acc[a].buffer);
     t_tidy(c, B);
-    const uint32_t from = B.n;
+    uint32_t from = B.n;
+    // a local chunk's region has a producer that no other entry has, unless
+    // another accessor writes the buffer too: it merges with nothing. So only
+    // what follows is probed, where the subtraction left no pieces before it
+    // (a probe of the table per chunk took half of a wave task's update)
+    bool only = true;
+    for (uint32_t o = 0; o < na; ++o)
+      if (o != a && (t.acc[o].mode & IGS_WRITE) && t.acc[o].buffer == t.acc[a].buffer) only = false;
     if (union_is_image(t, a, bd)) {
       // all chunks' writes form the image of the task's range: one subtraction
       Bx all;
@@ -3360,6 +3375,13 @@ __device__ __noinline__ void p5_state(Ctx& c, const igs_task& t, const Table& CH
         if (t_key(NB, m) != DEAD) all = bx_union(all, t_box(NB, m));
       const Bx U = map_box(t.acc[a], all, bd);
       if (!bx_empty(U)) t_subtract(c, B, NONE, U);
+      if (B.n != from) only = false;
+      if (B.live == 0 && !c.err) {  // nothing outside the written region: start afresh
+        B.n = 0;
+        from = 0;
+        t_publish(c, B);
+        __syncwarp();
+      }
       for (uint32_t base = 0; base < CH.n; base += 32) {
         const uint32_t slot = base + laneid();
         bool hit = false;
@@ -3375,6 +3397,7 @@ __device__ __noinline__ void p5_state(Ctx& c, const igs_task& t, const Table& CH
         if (!t_claim_ok(c, B, hit, s)) return;
         if (hit) t_put(B, s, 0, x, kid, mem, 1u << mem);
       }
+      if (only) from = B.n;
       for (uint32_t m = 0; m < c.N; ++m) {
         if (m == c.node || t_key(NB, m) == DEAD) continue;
         const Bx x = map_box(t.acc[a], t_box(NB, m), bd);
@@ -4139,6 +4162,7 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
   // this phase only add up-to-date memories and leave producers unchanged, so
   // a consumer with nothing stale now has nothing stale when its turn comes.
   Table& PC = c.s[S_CL];
+  const Table SB = c.s[S_T4];  // by PC entry: the bounding box of what is stale
   t_reset(PC);
   {
     const uint32_t total = CH.n * na;
@@ -4146,7 +4170,9 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
       const uint32_t i = base + laneid();
       bool hit = false;
       uint32_t flags = 0;
-      Bx x{};
+      Bx x{}, sb;
+      sb.lo[0] = sb.lo[1] = sb.lo[2] = 0xFFFFFFFFu;
+      sb.hi[0] = sb.hi[1] = sb.hi[2] = 0;
       if (i < total) {
         const uint32_t slot = i / na, a = i % na;
         if (t_v(CH, 0, slot) == c.node && (t.acc[a].mode & IGS_READ)) {
@@ -4162,8 +4188,12 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
 #pragma unroll
               for (uint32_t u = 0; u < 4; ++u) {
                 if (e[u].key == DEAD || !bx_overlap(e[u].b, x)) continue;
-                if (e[u].v0 == NONE) flags |= 1u;
-                else if (!((e[u].v2 >> m) & 1u)) flags |= 2u;
+                if (e[u].v0 == NONE) {
+                  flags |= 1u;
+                } else if (!((e[u].v2 >> m) & 1u)) {
+                  flags |= 2u;
+                  sb = bx_union(sb, bx_isect(e[u].b, x));
+                }
               }
             }
           }
@@ -4171,14 +4201,20 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
       }
       uint32_t s;
       if (!s_claim_ok(c, PC, hit, s)) return;
-      if (hit) t_put(PC, s, flags, x, i, 0, 0);
+      if (hit) {
+        t_put(PC, s, flags, x, i, 0, 0);
+        t_put(SB, s, 0, sb, 0, 0, 0);
+      }
     }
     __syncwarp();
   }
   // stale consumers that more than one worker would plan: shared by the
-  // helper warps. A consumer whose region meets no other stale consumer of
-  // its (buffer, memory) sees none of their copies, so it goes to the next
-  // worker in turn; the others are planned in order by their pair's worker.
+  // helper warps. A consumer whose stale part (its bounding box) meets that of
+  // no other consumer of its (buffer, memory) sees none of their copies, so it
+  // goes to the next worker in turn; the others are planned in order by their
+  // pair's worker. (Neighbouring chunks of a device overlap in their halos,
+  // but each misses only the row beyond the device: compared by their whole
+  // regions, one worker planned both.)
   bool multi = false;
   if (c.block && c.workers > 1 && c.nd->helper_scratch && !c.nd->stage_d2d) {
     for (uint32_t base = 0; base < PC.n; base += 32) {
@@ -4197,11 +4233,11 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
       const uint32_t mask = __ballot_sync(FULL, stale);
       if (stale) {
         const uint32_t b = FLD(PC, F_P4_BUF, k), m = FLD(PC, F_P4_WM, k) >> 8;
-        const Bx x = t_box(PC, k);
+        const Bx x = t_box(SB, k);
         bool alone = true;
         for (uint32_t o = 0; o < PC.n && alone; ++o)
           if (o != k && (t_key(PC, o) & 2u) && FLD(PC, F_P4_BUF, o) == b && (FLD(PC, F_P4_WM, o) >> 8) == m &&
-              bx_overlap(t_box(PC, o), x))
+              bx_overlap(t_box(SB, o), x))
             alone = false;
         const uint32_t w = alone ? (turn + __popc(mask & lanemask_lt())) % c.workers : p4_worker(b, m, c.D, c.workers);
         FLD(PC, F_P4_WM, k) = w | (m << 8);
