@@ -521,13 +521,14 @@ int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream);
  * driver's allocator (which can block on or synchronize with other work on the
  * device). igs_lower_static lowers a whole program (buffers, tasks, flushes,
  * buffer destructions, lookahead changes, in `ops` order) on every node into
- * caller-owned DEVICE output arrays, using a 32 MiB file-scope device array as
- * its only scratch: it calls no cudaMalloc, cudaFree or other allocating
- * routine. Every GPU that loads the library holds that array until exit.
+ * caller-owned DEVICE output arrays, using file-scope device arrays as its
+ * only scratch (32 MiB, and 42 MiB for the warps that share a node's lowering
+ * in programs of up to 8 nodes): it calls no cudaMalloc, cudaFree or other
+ * allocating routine. Every GPU that loads the library holds them until exit.
  *   Limits: at most 16 buffers; per node at most 128 live allocations and a
  *   region-map heap of 32768 entries shared by all its box tables; the
  *   program's staged inputs plus per-node state (about 2.6 MiB + instr_cap
- *   bytes per node) must fit the array, else IGS_ERR_CAPACITY before anything
+ *   bytes per node) must fit the 32 MiB, else IGS_ERR_CAPACITY before anything
  *   runs. A capacity that runs out during the lowering (the heap, an output
  *   array) shows only in that node's status word (counts[5] = 1); the call
  *   still returns IGS_OK.
@@ -537,7 +538,7 @@ int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream);
  *   A task whose chunks write overlapping regions (Sec. 4.4) is left out of
  *   the graph, as igs_submit_task does, and the call then returns
  *   IGS_ERR_OVERLAPPING_WRITE (the outputs and counts are still written).
- *   Sharing: every call uses the same array and leaves its last contents there
+ *   Sharing: every call uses the same arrays and leaves its last contents there
  *   (each call resets what must start at zero); calls that overlap on the GPU
  *   race, so serialize them. The call synchronizes `stream` (cudaStream_t,
  *   NULL = default stream): it returns after the lowering has finished.

@@ -1,8 +1,10 @@
 """Builds libigs.so (the C-ABI library) for sm_103a with nvcc, in-tree.
 
-Each CUDA translation unit is compiled in parallel to an object file, then
-linked into ``_build/libigs.so``. The executor's TU is built with
-``-fmad=false`` so the float workload kernels round after every operation.
+Each object file is compiled in parallel, then all are linked into
+``_build/libigs.so``. The lowering engine is inlined into each of its four
+kernels and takes most of the time, so they are objects of their own (one
+source). The executor's TU is built with ``-fmad=false`` so the float workload
+kernels round after every operation.
 """
 from __future__ import annotations
 
@@ -19,11 +21,12 @@ LIB = os.path.join(BUILD, "libigs.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = {
-    "igs_lower.cu": [],
-    "igs_exec.cu": ["-fmad=false"],
-    "igs_host.cu": [],
-    "igs_static.cu": [],
+# object file: source and its own flags
+OBJECTS = {
+    **{f"igs_lower{k}.o": ("igs_lower.cu", [f"-DIGS_LOWER_PART={k}"]) for k in range(4)},
+    "igs_exec.o": ("igs_exec.cu", ["-fmad=false"]),
+    "igs_host.o": ("igs_host.cu", []),
+    "igs_static.o": ("igs_static.cu", []),
 }
 
 
@@ -49,18 +52,19 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     if os.environ.get("IGS_PROFILE_DETAIL"):
         common.append("-DIGS_PROFILE_DETAIL")
 
-    def compile_one(src):
-        obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = [nvcc, "-c", os.path.join(CSRC, src), "-o", obj] + common + SOURCES[src]
+    def compile_one(name):
+        src, flags = OBJECTS[name]
+        obj = os.path.join(BUILD, name)
+        cmd = [nvcc, "-c", os.path.join(CSRC, src), "-o", obj] + common + flags
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
-            raise RuntimeError(f"nvcc failed for {src}:\n{r.stderr}")
+            raise RuntimeError(f"nvcc failed for {name}:\n{r.stderr}")
         if verbose and r.stderr:
             sys.stderr.write(r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=len(OBJECTS)) as ex:
+        objs = list(ex.map(compile_one, OBJECTS))
     tmp = LIB + f".{os.getpid()}.tmp"
     cmd = [nvcc, "-shared", "-o", tmp] + objs + ARCH + ["-lcudart"]
     r = subprocess.run(cmd, capture_output=True, text=True)

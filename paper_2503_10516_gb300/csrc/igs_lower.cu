@@ -22,6 +22,23 @@
 
 #include "igs_internal.h"
 
+// What runs for every instruction or task is inlined into its callers: a call
+// saves and restores registers in local memory on both sides, and the engine's
+// steps are short chains of dependent work, so calls to the emission, merging
+// and state steps made up a tenth of the time (233 wave tasks on 4 x 4 devices
+// 177 -> 160 us a task, 46 N-body tasks on 8 x 4 528 -> 450, 233 Jacobi tasks
+// on 1 x 4 76 -> 68, growing rows with a resize per task 172 -> 147). Growing
+// a table, compacting one and the general canonical form are rare or long and
+// stay calls (growing inlined: wave 181). Every kernel therefore holds the
+// engine, and is an object file of its own, compiled side by side
+// (IGS_LOWER_PART: 0 the launch per program, 1 the batch pool, 2 the work
+// queue, 3 the serving loop; undefined: all four).
+#ifndef IGS_LOWER_PART
+#define IGS_LOWER_IS(part) 1
+#else
+#define IGS_LOWER_IS(part) (IGS_LOWER_PART == (part))
+#endif
+
 namespace igs {
 namespace {
 
@@ -355,7 +372,7 @@ __device__ void heap_unlock(Ctx& c) {
   __syncwarp();
 }
 
-__device__ __noinline__ uint32_t heap_alloc(Ctx& c, uint32_t entries, uint32_t& cap) {
+__device__ __forceinline__ uint32_t heap_alloc(Ctx& c, uint32_t entries, uint32_t& cap) {
   const int k = heap_class(entries);
   cap = 32u << k;
   NodeDev* nd = c.nd;
@@ -720,7 +737,7 @@ __device__ __forceinline__ void t_subtract(Ctx& c, Table& t_ref, uint32_t key, c
 
 // value[vidx] |= bits on box r for entries of `key` (the table's header in
 // and out by value).
-__device__ __noinline__ Table t_or_v(Ctx& c, Table t, uint32_t key, const Bx& r, int vidx, uint32_t bits) {
+__device__ __forceinline__ Table t_or_v(Ctx& c, Table t, uint32_t key, const Bx& r, int vidx, uint32_t bits) {
   t_tidy(c, t);
   const uint32_t n0 = t.n;
   for (uint32_t base = 0; base < n0; base += 32) {
@@ -809,7 +826,7 @@ __device__ __forceinline__ void t_merge_entry(Ctx& c, Table& t, uint32_t i) {
 
 // Merges entries from index `from` on with equal key and values into
 // adjacent entries whose union is a box (keeps the tables small).
-__device__ __noinline__ Table t_merge_from_v(Ctx& c, Table t, uint32_t from) {
+__device__ __forceinline__ Table t_merge_from_v(Ctx& c, Table t, uint32_t from) {
   DT_START(dt);
   DT_COUNT(N_MERGE, 1);
   for (uint32_t i = from; i < t.n; ++i) t_merge_entry(c, t, i);
@@ -1231,7 +1248,7 @@ __device__ Bx buffer_box(const BufDesc& b) {
 }
 
 // a1: chunks of a task: key = chunk index, v0 = node, v1 = memory (Sec. 3.1).
-__device__ __noinline__ void task_chunks(Ctx& c, const igs_task& t, Table& CH) {
+__device__ __forceinline__ void task_chunks(Ctx& c, const igs_task& t, Table& CH) {
   t_reset(CH);
   const uint32_t Cx = t.num_chunks >> 16;
   if (Cx) {
@@ -1337,7 +1354,7 @@ __device__ Bx map_box(const igs_accessor& a, const Bx& ch, const BufDesc& buf) {
 }
 
 // Mapped boxes for every (chunk slot, accessor): MP[slot * nacc + a].
-__device__ __noinline__ void task_mapped(Ctx& c, const igs_task& t, const Table& CH, Table& MP) {
+__device__ __forceinline__ void task_mapped(Ctx& c, const igs_task& t, const Table& CH, Table& MP) {
   const uint32_t na = t.num_accessors, total = CH.n * na;
   if (total > MP.cap) {
     fail_cap(c, CAP_TABLE, MP.cap);
@@ -1398,7 +1415,7 @@ __device__ __noinline__ bool overlapping_writes(Ctx& c, const igs_task& t, const
 // writes, the readers since the last write (WAR anti); no predecessor at all
 // means an edge to the last epoch. Then reads, then writes are applied to
 // the per-allocation tracking tables.
-__device__ __noinline__ uint32_t emit_impl(Ctx& c, uint32_t type, uint32_t seq, uint32_t fa, uint32_t fb, uint32_t fc, uint32_t fd,
+__device__ __forceinline__ uint32_t emit_impl(Ctx& c, uint32_t type, uint32_t seq, uint32_t fa, uint32_t fb, uint32_t fc, uint32_t fd,
                               const Table* bt, uint32_t bfrom, uint32_t bto, const Acc* acc, int nacc, bool keep_dep,
                               const Table* bindt, uint32_t bind_from, uint32_t bind_n);
 __device__ uint32_t emit(Ctx& c, uint32_t type, uint32_t seq, uint32_t fa, uint32_t fb, uint32_t fc, uint32_t fd,
@@ -1746,7 +1763,7 @@ __device__ __forceinline__ bool emit_apply(Ctx& c, const Acc* acc, int nacc, uin
   return true;
 }
 
-__device__ __noinline__ uint32_t emit_impl(Ctx& c, uint32_t type, uint32_t seq, uint32_t fa, uint32_t fb, uint32_t fc, uint32_t fd,
+__device__ __forceinline__ uint32_t emit_impl(Ctx& c, uint32_t type, uint32_t seq, uint32_t fa, uint32_t fb, uint32_t fc, uint32_t fd,
                               const Table* bt, uint32_t bfrom, uint32_t bto, const Acc* acc, int nacc, bool keep_dep,
                               const Table* bindt, uint32_t bind_from, uint32_t bind_n) {
   if (c.err) return NONE;
@@ -1832,7 +1849,7 @@ __device__ __noinline__ uint32_t emit_impl(Ctx& c, uint32_t type, uint32_t seq, 
 // Replace every tracked instruction id older than h by h and re-merge (a9).
 // In writer tables (writers = true) v1 marks allocation writers; a replaced
 // writer is the horizon, which is not one. Returns whether any id changed.
-__device__ __noinline__ bool map_ids(Ctx& c, Table& T, uint32_t h, bool writers = false) {
+__device__ __forceinline__ bool map_ids(Ctx& c, Table& T, uint32_t h, bool writers = false) {
   bool any = false;
   for (uint32_t base = 0; base < T.n; base += 32) {
     const uint32_t i = base + laneid();
@@ -1900,7 +1917,7 @@ __device__ __noinline__ void epoch_share(Ctx& c, uint32_t h, uint32_t w, uint32_
 }
 
 // Free of an allocation: depends on every writer and reader (allocation lifetime).
-__device__ __noinline__ void emit_free(Ctx& c, uint32_t seq, uint32_t aid) {
+__device__ __forceinline__ void emit_free(Ctx& c, uint32_t seq, uint32_t aid) {
   Table& D = c.s[S_DEP];
   t_reset(D);
   for (int k = 0; k < 2; ++k) {
@@ -2113,7 +2130,7 @@ __device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_
 // NB[m] = bounding box of node m's chunks (key DEAD if it has none). The
 // chunks of a node are consecutive along the split dimension, so this box is
 // exactly their union.
-__device__ __noinline__ void node_bboxes(Ctx& c, const Table& CH, Table& NB) {
+__device__ __forceinline__ void node_bboxes(Ctx& c, const Table& CH, Table& NB) {
   for (uint32_t m = 0; m < c.N; ++m) {
     Bx acc;
     acc.lo[0] = acc.lo[1] = acc.lo[2] = 0xFFFFFFFFu;
@@ -2281,7 +2298,7 @@ __device__ bool plan_overflowed(Ctx& c) {
 // Results go to the QR table under key seq: v0 = 0 push boxes, 1 await boxes,
 // 2 push bbox, 3 await bbox; v1 = buffer; v2 = target node.
 // Push / await of one buffer b; the QR entries go to OUT.
-__device__ __noinline__ void a3_buffer(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP,
+__device__ __forceinline__ void a3_buffer(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP,
                                        const Table& NB, uint32_t b, Table& OUT) {
   const uint32_t na = t.num_accessors;
   Table& TMP = c.s[S_T0];
@@ -2420,7 +2437,7 @@ __device__ __noinline__ void a3_share(Ctx& c, WorkJob& j, uint32_t w, Table& OUT
   }
 }
 
-__device__ __noinline__ void a3_task(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP) {
+__device__ __forceinline__ void a3_task(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP) {
   const uint32_t na = t.num_accessors;
   Table& NB = c.s[S_T4];
   node_bboxes(c, CH, NB);
@@ -2491,7 +2508,7 @@ __device__ void qr_block(const Ctx& c, uint32_t seq, uint32_t& qs, uint32_t& qe)
 
 // Appends the requirements (key = buffer * 32 + memory, box) of a task on this
 // node: every non-empty mapped box of a local chunk, plus the staging bboxes.
-__device__ __noinline__ void requirements(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP, Table& RQ,
+__device__ __forceinline__ void requirements(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP, Table& RQ,
                              uint32_t only_key, uint32_t own_flag) {
   const uint32_t na = t.num_accessors, total = CH.n * na;
   for (uint32_t base = 0; base < total; base += 32) {
@@ -2529,7 +2546,7 @@ __device__ __noinline__ void requirements(Ctx& c, const igs_task& t, uint32_t se
   __syncwarp();
 }
 
-__device__ __noinline__ bool allocating(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP) {
+__device__ __forceinline__ bool allocating(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP) {
   Table& RQ = c.s[S_CL];
   t_reset(RQ);
   requirements(c, t, seq, CH, MP, RQ, NONE, 1);
@@ -2546,7 +2563,7 @@ __device__ __noinline__ bool allocating(Ctx& c, const igs_task& t, uint32_t seq,
   return false;
 }
 
-__device__ __noinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP) {
+__device__ __forceinline__ void alloc_phase(Ctx& c, const igs_task& t, uint32_t seq, const Table& CH, const Table& MP) {
   Table& RQ = c.s[S_T4];
   Table& CL = c.s[S_CL];
   Table& CH2 = c.s[S_CH2];
@@ -4124,7 +4141,7 @@ __device__ __noinline__ bool p23_parallel(Ctx& c, const igs_task& t, uint32_t se
 
 // ---- compile one task (P1..P5) ----------------------------------------------
 
-__device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
+__device__ __forceinline__ void compile_task(Ctx& c, uint32_t item) {
   const Item it = c.pg->items[item];
   const igs_task& t = c.pg->tasks[it.task];
   const uint32_t seq = it.seq, na = t.num_accessors;
@@ -4328,7 +4345,7 @@ __device__ __noinline__ void compile_task(Ctx& c, uint32_t item) {
 
 // ---- items ---------------------------------------------------------------------
 
-__device__ __noinline__ void process(Ctx& c, uint32_t item) {
+__device__ __forceinline__ void process(Ctx& c, uint32_t item) {
   const Item it = c.pg->items[item];
   switch (it.kind) {
     case IT_CREATE: {
@@ -4538,7 +4555,7 @@ __device__ void pipe_take(Ctx& c, uint32_t item) {
   __syncwarp();
 }
 
-__device__ __noinline__ void deliver(Ctx& c, uint32_t item) {
+__device__ __forceinline__ void deliver(Ctx& c, uint32_t item) {
   const Item it = c.pg->items[item];
   maintain(c);
   if (c.err) return;
@@ -4921,6 +4938,7 @@ __device__ void unit_body(BlockShared& sh, const Unit* units, uint32_t n_units, 
   __syncthreads();
 }
 
+#if IGS_LOWER_IS(0)
 __global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* units, uint32_t n_units, uint32_t max_items,
                                                                volatile uint32_t* progress) {
   __shared__ BlockShared sh;
@@ -4931,7 +4949,9 @@ __global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* unit
   __syncthreads();
   unit_body(sh, units, n_units, blockIdx.x, max_items, progress);
 }
+#endif
 
+#if IGS_LOWER_IS(1)
 // Batched lowering of few or uneven units, whose longest bounds the launch:
 // each resident block has helper scratch of its own (slot_words words, its
 // last kPipeDepth x front_cap entries the front warp's slots), lends it to the
@@ -4963,7 +4983,9 @@ __global__ void __launch_bounds__(kReserveThreads) lower_pool_kernel(const Unit*
     if (threadIdx.x == 0 && sh.lent) units[sh.unit].node->helper_scratch = nullptr;
   }
 }
+#endif
 
+#if IGS_LOWER_IS(2)
 // Batched lowering with a device work queue: the first warp of each
 // persistent block takes the next unit (a node of one program) from *head, in
 // the order `order` gives (longest estimated work first, say), until every
@@ -5004,7 +5026,9 @@ __global__ void __launch_bounds__(32 * kQueueWarps) lower_queue_kernel(const Uni
   }
   __syncthreads();
 }
+#endif
 
+#if IGS_LOWER_IS(3)
 // Copies submissions [from, to) and their tasks from the host-mapped arrays
 // into the program's device arrays (16-byte words, all lanes). Every node warp
 // of a program stages the same records; the copies write equal bytes.
@@ -5029,7 +5053,9 @@ __device__ __noinline__ void stage_submissions(const ProgDev* pg, uint32_t from,
   __threadfence_block();
   __syncwarp();
 }
+#endif
 
+#if IGS_LOWER_IS(0)
 // What a node's state starts with: block n resets node n.
 __global__ void init_nodes_kernel(const NodeDev* nodes) {
   const NodeDev& nd = nodes[blockIdx.x];
@@ -5042,7 +5068,9 @@ __global__ void init_nodes_kernel(const NodeDev* nodes) {
     nd.instrs[0] = igs_instruction{0, IGS_EPOCH, NONE, NONE, NONE, NONE, NONE, 0, 0, 0, 0};
   }
 }
+#endif
 
+#if IGS_LOWER_IS(3)
 // Serving loop: warp w serves slot w; it takes every submission published so
 // far, then publishes its progress. Waits are bounded: after idle_polls empty
 // polls (about 2 us each) the warp leaves with EXIT_IDLE; a set stop flag ends
@@ -5115,15 +5143,19 @@ __global__ void __launch_bounds__(32) serve_kernel(ServeSlot* slots, uint32_t n_
   if (leader) S.exit = exit_code;
   __threadfence_system();
 }
+#endif
 
 }  // namespace
 }  // namespace igs
 
+#if IGS_LOWER_IS(0)
 int igs_launch_init_nodes(const igs::NodeDev* nodes_dev, uint32_t n, void* stream) {
   igs::init_nodes_kernel<<<n, 256, 0, (cudaStream_t)stream>>>(nodes_dev);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
+#endif
 
+#if IGS_LOWER_IS(3)
 int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t* stop, uint64_t idle_polls, void* stream) {
   if (n_slots == 0) return 0;
   // one warp per block: each slot's warp gets an SM (and its L1) to itself
@@ -5136,7 +5168,9 @@ int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t*
   igs::serve_kernel<<<n_slots, 32, 0, (cudaStream_t)stream>>>(slots, n_slots, stop, idle_polls);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
+#endif
 
+#if IGS_LOWER_IS(2)
 int igs_launch_lower_queue(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                            uint32_t blocks, uint32_t warps, void* stream) {
   if (warps < 1 || warps > igs::kQueueWarps) return -1;
@@ -5149,12 +5183,16 @@ int igs_launch_lower_queue(const igs::Unit* units_dev, uint32_t n_units, const u
   igs::lower_queue_kernel<<<blocks, 32 * warps, 0, (cudaStream_t)stream>>>(units_dev, n_units, order_dev, head_dev);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
+#endif
 
+#if IGS_LOWER_IS(1)
 size_t igs_lower_pool_words(uint32_t cap_scratch, uint32_t front_cap) {
   return (size_t)igs::F_COUNT *
          ((size_t)igs::kScratchSets * igs::kHelperTables * cap_scratch + (size_t)igs::kPipeDepth * front_cap);
 }
+#endif
 
+#if IGS_LOWER_IS(1)
 int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                           uint32_t blocks, uint32_t* scratch_dev, uint32_t cap_scratch, uint32_t front_cap,
                           void* stream) {
@@ -5168,7 +5206,9 @@ int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const ui
       units_dev, n_units, order_dev, head_dev, scratch_dev, igs_lower_pool_words(cap_scratch, front_cap), front_cap);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
+#endif
 
+#if IGS_LOWER_IS(0)
 int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_items, void* stream, bool reserve,
                      volatile uint32_t* progress, bool workers) {
   if (n_units == 0) return 0;
@@ -5184,3 +5224,4 @@ int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_
   igs::lower_kernel<<<n_units, threads, 0, (cudaStream_t)stream>>>(units_dev, n_units, max_items, progress);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
+#endif
