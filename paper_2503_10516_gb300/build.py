@@ -1,7 +1,7 @@
 """Builds libigs.so (the C-ABI library) for sm_103a with nvcc, in-tree.
 
 Each object file is compiled in parallel, then all are linked into
-``_build/libigs.so``. The lowering engine is inlined into each of its four
+``_build/libigs.so``. The lowering engine is inlined into each of its
 kernels and takes most of the time, so they are objects of their own (one
 source). The executor's TU is built with ``-fmad=false`` so the float workload
 kernels round after every operation.
@@ -23,7 +23,7 @@ INCLUDE = os.path.join(ROOT, "include")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # object file: source and its own flags
 OBJECTS = {
-    **{f"igs_lower{k}.o": ("igs_lower.cu", [f"-DIGS_LOWER_PART={k}"]) for k in range(4)},
+    **{f"igs_lower{k}.o": ("igs_lower.cu", [f"-DIGS_LOWER_PART={k}"]) for k in range(5)},
     "igs_exec.o": ("igs_exec.cu", ["-fmad=false"]),
     "igs_host.o": ("igs_host.cu", []),
     "igs_static.o": ("igs_static.cu", []),

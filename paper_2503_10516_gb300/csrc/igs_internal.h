@@ -246,6 +246,9 @@ int igs_launch_init_nodes(const igs::NodeDev* nodes_dev, uint32_t n, void* strea
 // node's kernel phase (when the node has helper scratch).
 int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_items, void* stream,
                      bool reserve = false, volatile uint32_t* progress = nullptr, bool workers = false);
+// One block of one warp per unit.
+int igs_launch_lower_alone(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_items, void* stream,
+                           volatile uint32_t* progress);
 // Persistent serving loop over n_slots slots; exits when *stop is set or a
 // warp stays idle for idle_polls polls (about 2 us each).
 int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t* stop, uint64_t idle_polls, void* stream);

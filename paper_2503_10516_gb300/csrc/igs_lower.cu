@@ -32,7 +32,7 @@
 // stay calls (growing inlined: wave 181). Every kernel therefore holds the
 // engine, and is an object file of its own, compiled side by side
 // (IGS_LOWER_PART: 0 the launch per program, 1 the batch pool, 2 the work
-// queue, 3 the serving loop; undefined: all four).
+// queue, 3 the serving loop, 4 one-warp blocks; undefined: all).
 #ifndef IGS_LOWER_PART
 #define IGS_LOWER_IS(part) 1
 #else
@@ -1946,7 +1946,7 @@ __device__ __forceinline__ void emit_free(Ctx& c, uint32_t seq, uint32_t aid) {
 // neither the buffer state nor the allocation tables change; the regions its
 // earlier copies of b into memory m cover count as up to date, as they would
 // after those copies' buffer-state update.
-__device__ __noinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_t m, uint32_t dst, const Table& T, uint32_t from,
+__device__ __forceinline__ void coherence(Ctx& c, uint32_t seq, uint32_t b, uint32_t m, uint32_t dst, const Table& T, uint32_t from,
                           uint32_t to) {
   Table& Q = c.s[S_T0];
   Table& G = c.s[S_T1];
@@ -4884,11 +4884,15 @@ __device__ void lower_unit(const Unit* units, uint32_t n_units, uint32_t max_ite
   if (pr) publish_progress(c, pr, cursor);
 }
 
-// Block b lowers unit b with its first warp. Blocks launched with more warps
-// (kReserveThreads) park the others at the barrier: they hold most of the
-// SM's registers, so no block of another kernel (the executor's copies and
+// Block b lowers unit b. A block of several warps has helper and front warps
+// and an SM to itself, so it is compiled for as many registers as 384 threads
+// leave (168); launched with all 384, its other warps park at the barrier and
+// hold the rest, so no block of another kernel (the executor's copies and
 // kernels running concurrently) shares the SM, its issue slots or its L1.
-constexpr uint32_t kReserveThreads = 512;
+// With 128 registers (512 threads) 233 wave tasks on 4 x 4 devices took 156 us
+// a task, now 152; 46 N-body tasks on 8 x 4 443, now 424. One-warp blocks, of
+// which an SM holds as many as its registers allow, keep to 128.
+constexpr uint32_t kReserveThreads = 384, kAloneThreads = 512;
 // Thread 0: a block's shared state before it lowers unit u: a front warp when
 // the block has one, the node has its scratch set and the launch lowers
 // several items.
@@ -4938,9 +4942,10 @@ __device__ void unit_body(BlockShared& sh, const Unit* units, uint32_t n_units, 
   __syncthreads();
 }
 
-#if IGS_LOWER_IS(0)
-__global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* units, uint32_t n_units, uint32_t max_items,
-                                                               volatile uint32_t* progress) {
+#if IGS_LOWER_IS(0) || IGS_LOWER_IS(4)
+template <uint32_t kThreads>
+__global__ void __launch_bounds__(kThreads, 1) lower_kernel(const Unit* units, uint32_t n_units, uint32_t max_items,
+                                                           volatile uint32_t* progress) {
   __shared__ BlockShared sh;
   if (threadIdx.x == 0) {
     sh.lent = 0;
@@ -4956,7 +4961,7 @@ __global__ void __launch_bounds__(kReserveThreads) lower_kernel(const Unit* unit
 // each resident block has helper scratch of its own (slot_words words, its
 // last kPipeDepth x front_cap entries the front warp's slots), lends it to the
 // node it lowers, and takes units longest first from *head.
-__global__ void __launch_bounds__(kReserveThreads) lower_pool_kernel(const Unit* units, uint32_t n_units,
+__global__ void __launch_bounds__(kReserveThreads, 1) lower_pool_kernel(const Unit* units, uint32_t n_units,
                                                                     const uint32_t* order, uint32_t* head,
                                                                     uint32_t* scratch, size_t slot_words,
                                                                     uint32_t front_cap) {
@@ -5208,20 +5213,34 @@ int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const ui
 }
 #endif
 
+// Carveout: each node's tables share an L1 with as few other units as
+// possible (one unit per block, so that units spread over the SMs).
+#if IGS_LOWER_IS(4)
+int igs_launch_lower_alone(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_items, void* stream,
+                           volatile uint32_t* progress) {
+  static bool carveout = false;
+  if (!carveout) {
+    cudaFuncSetAttribute(igs::lower_kernel<igs::kAloneThreads>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    carveout = true;
+  }
+  igs::lower_kernel<igs::kAloneThreads><<<n_units, 32, 0, (cudaStream_t)stream>>>(units_dev, n_units, max_items, progress);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+#endif
 #if IGS_LOWER_IS(0)
 int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_items, void* stream, bool reserve,
                      volatile uint32_t* progress, bool workers) {
   if (n_units == 0) return 0;
-  // one unit per block, so that units spread over the SMs (each node's
-  // tables then share an L1 with as few other units as possible)
+  if (!reserve && !workers) return igs_launch_lower_alone(units_dev, n_units, max_items, stream, progress);
   static bool carveout = false;
   if (!carveout) {
-    cudaFuncSetAttribute(igs::lower_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(igs::lower_kernel<igs::kReserveThreads>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
     carveout = true;
   }
-  // with workers: kMaxWorkers warps plus the front warp of pipelined launches
-  const uint32_t threads = reserve ? igs::kReserveThreads : (workers ? 32 * (igs::kMaxWorkers + 1) : 32);
-  igs::lower_kernel<<<n_units, threads, 0, (cudaStream_t)stream>>>(units_dev, n_units, max_items, progress);
+  // kMaxWorkers warps plus the front warp of pipelined launches
+  const uint32_t threads = reserve ? igs::kReserveThreads : 32 * (igs::kMaxWorkers + 1);
+  igs::lower_kernel<igs::kReserveThreads><<<n_units, threads, 0, (cudaStream_t)stream>>>(units_dev, n_units, max_items,
+                                                                                        progress);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 #endif
