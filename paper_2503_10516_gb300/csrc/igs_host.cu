@@ -892,7 +892,7 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
   // lowers a unit about twice as fast as one warp, but takes an SM that about
   // ten one-warp blocks share: it is the better form while twice the SMs'
   // pace gets through all units well before one warp gets through the longest
-  // (24 uneven programs of 142 nodes: 259 ms with one warp per node, 126 ms).
+  // (24 uneven programs of 142 nodes: 259 ms with one warp per node, 91 ms).
   uint32_t* pool = nullptr;
   uint32_t pool_blocks = 0, pool_cap = 32, front_cap = 0;
   if (!shape) {

@@ -286,7 +286,7 @@ extern "C" int igs_lower_static(const igs_config* cfg, const igs_static_buffer* 
   uint32_t result[64];  // {status, rejected tasks} per node
   // Each node is lowered by its block's helper and front
   // warps together (one warp per node took 15.4 ms for 28 wave tasks on 4 x 4
-  // devices in 64 chunks, the shared form 7.7 ms). Their staging and the
+  // devices in 64 chunks, the shared form 4.9 ms). Their staging and the
   // slabs they place may run out where a single warp's do not, so whatever
   // does not come out well is lowered again, from the start, by one warp.
   for (int helped = N <= kHelpedNodes ? 1 : 0; helped >= 0; --helped) {
