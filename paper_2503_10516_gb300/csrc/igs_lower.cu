@@ -2229,9 +2229,10 @@ struct BlockShared {
   WorkJob job;
   uint32_t piped;
   Pipe pipe;
-  // blocks of a batch with helper scratch of their own: the unit being
-  // lowered, and whether its node uses that scratch
+  // blocks of a batch with helper scratch of their own (lent set): the unit
+  // being lowered, and the scratch its node had
   uint32_t unit, lent;
+  uint32_t* own;
 };
 
 __device__ __forceinline__ void worker_bar(uint32_t workers) {
@@ -4973,19 +4974,18 @@ __global__ void __launch_bounds__(kReserveThreads, 1) lower_pool_kernel(const Un
       sh.unit = i < n_units ? order[i] : NONE;
       if (sh.unit != NONE) {
         const Unit u = units[sh.unit];
-        sh.lent = u.node->helper_scratch == nullptr;
-        if (sh.lent) u.node->helper_scratch = mine;
+        sh.lent = 1;
+        sh.own = u.node->helper_scratch;
+        u.node->helper_scratch = mine;
         unit_begin(sh, u, blockDim.x >> 5, NONE);
-        if (sh.lent) {
-          sh.pipe.qr = mine + slot_words - (size_t)kPipeDepth * front_cap * F_COUNT;
-          sh.pipe.qr_cap = front_cap;
-        }
+        sh.pipe.qr = mine + slot_words - (size_t)kPipeDepth * front_cap * F_COUNT;
+        sh.pipe.qr_cap = front_cap;
       }
     }
     __syncthreads();
     if (sh.unit == NONE) break;
     unit_body(sh, units, n_units, sh.unit, NONE, nullptr);
-    if (threadIdx.x == 0 && sh.lent) units[sh.unit].node->helper_scratch = nullptr;
+    if (threadIdx.x == 0) units[sh.unit].node->helper_scratch = sh.own;
   }
 }
 #endif

@@ -36,16 +36,20 @@ def _batch_is_the_oracles(progs, ctxs):
         c.close()
 
 
+@pytest.mark.parametrize("own", [False, True])
 @pytest.mark.parametrize("devices", [1, 2])
-def test_stages_too_small_for_the_plan(devices):
+def test_stages_too_small_for_the_plan(devices, own):
     """200 x 200 edges in 512-entry tables (2048 edges a worker): planned
-    kernels fall back to one warp."""
+    kernels fall back to one warp, also where the context has helper scratch of
+    its own from an earlier launch."""
     from paper_2503_10516_gb300 import igs
     p = _all_to_all(200, 1, devices)
     c = igs.Context(p.nodes, p.devices, p.horizon_step, p.lookahead, mode=igs.MODE_BATCHED, scratch_capacity=512)
     for op in p.ops:
         if op[0] == "buffer":
             c.create_buffer(op[1].dims, op[1].extent[:op[1].dims], op[1].elem_size, op[1].init)
+            if own:
+                c.sync()
         elif op[0] == "task":
             c.submit(op[1])
         else:
