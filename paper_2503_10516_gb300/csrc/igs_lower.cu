@@ -2225,7 +2225,8 @@ struct Pipe {
 
 struct BlockShared {
   int lock;
-  volatile uint32_t cmd, err, err_info;
+  volatile uint32_t cmd;
+  unsigned long long failed;  // the gravest failure_word of the shared phase (0: none)
   WorkJob job;
   uint32_t piped;
   Pipe pipe;
@@ -2259,6 +2260,20 @@ __device__ __forceinline__ Table scratch_table(uint32_t* base, uint32_t cap) {
   return t;
 }
 
+// A worker's failure in one word, graver ones larger: whether more is lost than
+// a plan that found no room in a stage or scratch table (planning: its share
+// changes no table), the status, what ran out. The workers' words are
+// collected by their maximum, so none hides behind a lesser one.
+__device__ __forceinline__ unsigned long long failure_word(const Ctx& c, bool planning) {
+  const bool room = planning && c.err == ST_CAPACITY && (c.err_info >> 24) == (uint32_t)CAP_TABLE;
+  return (room ? 0ull : 1ull << 63) | ((unsigned long long)c.err << 32) | c.err_info;
+}
+// Whether worker w's share of a phase changes no table: the coherence plan, and
+// the kernel plan except for its last worker (p4_states).
+__device__ __forceinline__ bool plans_only(uint32_t cmd, uint32_t w, uint32_t workers) {
+  return cmd == CMD_P4 || (cmd == CMD_P5_PLAN && w + 1 != workers);
+}
+
 // Posts a job (lane 0 has filled sh.job) and runs warp 0's share between the
 // start and end barriers; returns false on a failure of any worker.
 template <class F>
@@ -2266,29 +2281,31 @@ __device__ bool run_shared(Ctx& c, BlockShared& sh, uint32_t cmd, F share0) {
   __syncwarp();
   if (laneid() == 0) {
     c.nd->prof[31] += 1;  // shared phases run (profile counter)
-    sh.err = ST_OK;
+    sh.failed = 0;
     sh.cmd = cmd;
     __threadfence_block();
   }
   __syncwarp();
   worker_bar(c.workers);  // helpers start
   share0();
+  if (c.err != ST_OK && laneid() == 0) atomicMax(&sh.failed, failure_word(c, plans_only(cmd, 0, c.workers)));
   worker_bar(c.workers);  // every share done
-  if (sh.err != ST_OK && c.err == ST_OK) {
-    c.err = sh.err;
-    c.err_info = sh.err_info;
+  const unsigned long long f = sh.failed;
+  if (f) {
+    c.err = (uint32_t)(f >> 32) & 0x7FFFFFFFu;
+    c.err_info = (uint32_t)f;
   }
   return c.err == ST_OK;
 }
 
-// Whether a phase that only plans (no table has changed) failed for want of
-// room in a stage or scratch table: then, in blocks that lend their scratch
-// (calls that one warp used to serve), the failure is cleared, and the caller
-// takes the single-warp path, which stages nothing.
+// Whether the planners of the phase that just failed found no room in a stage
+// or scratch table and nothing else went wrong (the kernel plan's last worker
+// changes tables meanwhile: its failure stands): then, in blocks that lend
+// their scratch (calls that one warp used to serve), the failure is cleared,
+// and the caller takes the single-warp path, which stages nothing.
 __device__ bool plan_overflowed(Ctx& c) {
-  if (c.err != ST_CAPACITY || (c.err_info >> 24) != (uint32_t)CAP_TABLE ||
-      !static_cast<BlockShared*>(c.block)->lent)
-    return false;
+  const BlockShared& sh = *static_cast<BlockShared*>(c.block);
+  if (!sh.lent || sh.failed == 0 || (sh.failed >> 63)) return false;
   c.err = ST_OK;
   c.err_info = 0;
   return true;
@@ -3295,10 +3312,7 @@ __device__ void helper_loop(BlockShared& sh, uint32_t w, uint32_t workers) {
       if (laneid() == 0) {
         atomicAdd(reinterpret_cast<unsigned long long*>(&j.nd->map_reads), (unsigned long long)hc.map_reads);
         atomicAdd(reinterpret_cast<unsigned long long*>(&j.nd->map_writes), (unsigned long long)hc.map_writes);
-        if (hc.err != ST_OK) {
-          sh.err_info = hc.err_info;
-          sh.err = hc.err;
-        }
+        if (hc.err != ST_OK) atomicMax(&sh.failed, failure_word(hc, plans_only(cmd, w, j.workers)));
       }
       __syncwarp();
     }
@@ -4044,15 +4058,10 @@ __device__ __noinline__ bool p23_parallel(Ctx& c, const igs_task& t, uint32_t se
     j.workers = c.workers;
     j.p3_n = n;
   }
-  uint32_t own = ST_OK;
-  if (!run_shared(c, sh, CMD_P3, [&]() {
-        p2_pushes(c, seq, qs, qe);
-        own = c.err;
-      })) {
-    // the pushes are done: awaits whose plans did not fit follow them
-    if (own == ST_OK && plan_overflowed(c)) p3_awaits(c, t, seq, CH, MP, qs, qe);
-    return true;
-  }
+  // a stage has room for whatever fits the scratch tables of the single-warp
+  // path (its boxes are those of two tables, its edges of four), so there is
+  // nothing to fall back to
+  if (!run_shared(c, sh, CMD_P3, [&]() { p2_pushes(c, seq, qs, qe); })) return true;
   // the planned instructions in group order, each with the single-warp
   // path's table updates
   for (uint32_t gi = 0; gi < n && !c.err; ++gi) {
@@ -4900,7 +4909,7 @@ constexpr uint32_t kReserveThreads = 384, kAloneThreads = 512;
 __device__ void unit_begin(BlockShared& sh, const Unit& u, uint32_t warps, uint32_t max_items) {
   sh.lock = 0;
   sh.cmd = CMD_NONE;
-  sh.err = ST_OK;
+  sh.failed = 0;
   sh.piped = 0;
   const NodeDev* nd = u.node;
   if (warps <= kFrontWarp || !nd->helper_scratch || nd->status != ST_OK) return;
@@ -5005,7 +5014,7 @@ __global__ void __launch_bounds__(32 * kQueueWarps) lower_queue_kernel(const Uni
   if (threadIdx.x == 0) {
     sh.lock = 0;
     sh.cmd = CMD_NONE;
-    sh.err = ST_OK;
+    sh.failed = 0;
     sh.lent = 0;
   }
   __syncthreads();

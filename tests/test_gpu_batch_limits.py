@@ -1,0 +1,72 @@
+"""Batches at the edge of a context's capacities: a launch that lends its
+blocks' helper and front warps to the nodes answers as one warp per node does,
+whatever runs out where."""
+import pytest
+
+from paper_2503_10516_gb300 import workloads as W
+from tests.harness import assert_same_graph, oracle_graphs
+
+pytestmark = pytest.mark.gpu
+
+
+def _context(prog, **caps):
+    from paper_2503_10516_gb300 import igs
+    return igs.Context(prog.nodes, prog.devices, prog.horizon_step, prog.lookahead, mode=igs.MODE_BATCHED,
+                       max_instructions=8192, max_edges=1 << 18, max_boxes=1 << 15, max_queue=256, **caps)
+
+
+def _submit(c, ops):
+    for op in ops:
+        if op[0] == "buffer":
+            c.create_buffer(op[1].dims, op[1].extent[:op[1].dims], op[1].elem_size, op[1].init)
+        elif op[0] == "task":
+            c.submit(op[1])
+        elif op[0] == "destroy":
+            c.destroy_buffer(op[1])
+        else:
+            c.submit_epoch()
+
+
+def _lower(prog, parts, shape, **caps):
+    """The program's graphs, lowered by one batch per part of its operations;
+    None where a capacity ran out."""
+    from paper_2503_10516_gb300 import igs
+    c = _context(prog, **caps)
+    try:
+        for ops in parts:
+            _submit(c, ops)
+            igs.lower_batch([c], shape)
+        return [c.graph(n) for n in range(prog.nodes)]
+    except igs.IgsError as e:
+        assert e.code == igs.IGS_ERR_CAPACITY
+        return None
+    finally:
+        c.close()
+
+
+def _pieces_program():
+    """170 rows written on two devices. The kernels of the second task read
+    the inner columns of all rows: their edges (170 each) overflow the workers'
+    stages (1024 edges at 256 entries), while the up-to-date bits of the
+    copies, set beside that plan, split the rows' state into pieces. The last
+    task reads one such row whole, so it copies what the bits say."""
+    ext = (170, 4, 1)
+    ops = [("buffer", W.Buffer(2, ext, 4, None, "u32"))]
+    ops.append(("task", W.Task(2, ext, 170, W.K_NOP, [W.Accessor(0, W.WRITE, W.one_to_one())])))
+    for chunks, box in ((48, W.fixed_box((0, 1), (170, 3))), (2, W.fixed_box((84, 0), (85, 4)))):
+        ops.append(("task", W.Task(2, ext, chunks, W.K_NOP, [W.Accessor(0, W.READ, box)])))
+    return W.Program("pieces", 1, 2, 100, 1, ops)
+
+
+def test_state_table_runs_out_beside_an_overflowing_plan():
+    """Whichever table the heap runs out for while the kernel plan overflows
+    its stages: the lowering ends with a capacity error or is the oracle's."""
+    prog = _pieces_program()
+    ref, _ = oracle_graphs(prog)
+    done = []
+    for heap in range(2048, 4352, 64):
+        got = _lower(prog, [prog.ops], None, map_heap=heap, scratch_capacity=256)
+        if got is not None:
+            done.append(heap)
+            assert_same_graph(got[0], ref[0], f"heap of {heap} entries")
+    assert done and done[0] > 2048  # the range reaches from too small to enough
