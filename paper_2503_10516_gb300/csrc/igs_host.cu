@@ -2158,6 +2158,7 @@ extern "C" int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream) 
       if (j.box.lo[d] < j.src_box.lo[d] || j.box.hi[d] > j.src_box.hi[d] || j.box.lo[d] < j.dst_box.lo[d] ||
           j.box.hi[d] > j.dst_box.hi[d])
         return IGS_ERR_INVALID_ARG;
+    if (j.elem_size == 0) continue;  // no bytes (and no rows to split them into)
     if (!make_copy_job(static_cast<const uint8_t*>(j.src), j.src_box.lo, j.src_box.hi, static_cast<uint8_t*>(j.dst),
                        j.dst_box.lo, j.dst_box.hi, j.box, j.elem_size, J))
       continue;
