@@ -1055,9 +1055,13 @@ struct Pending {
 };
 
 // Collapses a box copy between two row-major allocations into rows of
-// contiguous bytes.
-bool make_copy_job(const uint8_t* src, const uint32_t slo[3], const uint32_t shi[3], uint8_t* dst, const uint32_t dlo[3],
-                   const uint32_t dhi[3], const igs_box& b, uint32_t elem, CopyJob& J) {
+// contiguous bytes and hands them to add(job): one job, or several where the
+// rows are longer than the jobs' 32-bit lengths take. False if the box is empty
+// or not inside both allocations.
+template <class F>
+bool make_copy_jobs(const uint8_t* src, const uint32_t slo[3], const uint32_t shi[3], uint8_t* dst,
+                    const uint32_t dlo[3], const uint32_t dhi[3], const igs_box& b, uint32_t elem, F add) {
+  CopyJob J{};
   uint64_t e[3], ss[3], ds[3];
   for (int d = 0; d < 3; ++d) {
     if (b.lo[d] >= b.hi[d]) return false;
@@ -1103,9 +1107,12 @@ bool make_copy_job(const uint8_t* src, const uint32_t slo[3], const uint32_t shi
     J.extent[0] = J.extent[1] = 1;
     J.src_stride[0] = J.dst_stride[0] = J.src_stride[1] = J.dst_stride[1] = 0;
   }
-  // very long runs are split into rows of at most 1 GiB to keep 32-bit lengths
-  J.extent[2] = (uint32_t)std::min<uint64_t>(run, 1ull << 30);
-  if (run > (1ull << 30)) return false;
+  // pieces of at most 1 GiB, which keep the rows' alignment
+  for (constexpr uint64_t kPiece = 1ull << 30; run; J.src += kPiece, J.dst += kPiece) {
+    J.extent[2] = (uint32_t)std::min(run, kPiece);
+    add(J);
+    run -= J.extent[2];
+  }
   return true;
 }
 
@@ -1687,13 +1694,13 @@ int exec_walk(igs_ctx* c, Pending& p, cudaStream_t xs, bool* halted_any, bool* p
               ExecAlloc* d = get_alloc(c, n, in.b, in.c);
               if (!s || !d) return fail_ctx(c, IGS_ERR_STATE, "copy between unknown allocations");
               const uint32_t F = g ? flow_node(n, i, FK_COPY) : 0;
-              for (uint32_t k = 0; k < in.box_cnt; ++k) {
-                CopyJob J{};
-                if (!make_copy_job(s->ptr, s->lo, s->hi, d->ptr, d->lo, d->hi, h.boxes[in.box_off + k], c->bufs[in.c].elem, J))
+              for (uint32_t k = 0; k < in.box_cnt; ++k)
+                if (!make_copy_jobs(s->ptr, s->lo, s->hi, d->ptr, d->lo, d->hi, h.boxes[in.box_off + k],
+                                    c->bufs[in.c].elem, [&](const CopyJob& J) {
+                                      if (g) g->add_copy(F, J);
+                                      else add_copy(p, L + 1, J);
+                                    }))
                   return fail_ctx(c, IGS_ERR_STATE, "bad copy box");
-                if (g) g->add_copy(F, J);
-                else add_copy(p, L + 1, J);
-              }
               h.level[i] = L + 1;
               break;
             }
@@ -1711,15 +1718,13 @@ int exec_walk(igs_ctx* c, Pending& p, cudaStream_t xs, bool* halted_any, bool* p
               uint64_t bytes = elem;
               for (int d = 0; d < 3; ++d) bytes *= sr.box.hi[d] - sr.box.lo[d];
               CK(cudaMallocAsync((void**)&sr.mail, bytes ? bytes : 1, xs));
-              CopyJob J{};
-              if (!make_copy_job(sa->ptr, sa->lo, sa->hi, sr.mail, sr.box.lo, sr.box.hi, sr.box, elem, J))
+              if (g) sr.fid = flow_node(n, i, FK_COPY);
+              if (!make_copy_jobs(sa->ptr, sa->lo, sa->hi, sr.mail, sr.box.lo, sr.box.hi, sr.box, elem,
+                                  [&](const CopyJob& J) {
+                                    if (g) g->add_copy(sr.fid, J);
+                                    else add_copy(p, L + 1, J);
+                                  }))
                 return fail_ctx(c, IGS_ERR_STATE, "bad send box");
-              if (g) {
-                sr.fid = flow_node(n, i, FK_COPY);
-                g->add_copy(sr.fid, J);
-              } else {
-                add_copy(p, L + 1, J);
-              }
               c->sends.insert({key_of(in.seq, in.c, in.b), sr});
               h.level[i] = L + 1;
               break;
@@ -1761,11 +1766,10 @@ int exec_walk(igs_ctx* c, Pending& p, cudaStream_t xs, bool* halted_any, bool* p
                 auto& parts = split_parts[((uint64_t)n << 32) | i];
                 for (auto it = range.first; it != range.second; ++it) {
                   const igs_box& b = it->second.box;
-                  CopyJob J{};
-                  if (!make_copy_job(it->second.mail, b.lo, b.hi, d->ptr, d->lo, d->hi, b, c->bufs[in.c].elem, J))
-                    return fail_ctx(c, IGS_ERR_STATE, "bad receive box");
                   const uint32_t cf = g->add_node(FK_COPY);
-                  g->add_copy(cf, J);
+                  if (!make_copy_jobs(it->second.mail, b.lo, b.hi, d->ptr, d->lo, d->hi, b, c->bufs[in.c].elem,
+                                      [&](const CopyJob& J) { g->add_copy(cf, J); }))
+                    return fail_ctx(c, IGS_ERR_STATE, "bad receive box");
                   g->edges.push_back({gate, cf});
                   if (it->second.call == c->exec_call) g->edges.push_back({it->second.fid, cf});
                   g->edges.push_back({cf, sid});
@@ -1783,16 +1787,14 @@ int exec_walk(igs_ctx* c, Pending& p, cudaStream_t xs, bool* halted_any, bool* p
               }
               for (auto it = range.first; it != range.second; ++it) {
                 const igs_box& b = it->second.box;
-                CopyJob J{};
-                if (!make_copy_job(it->second.mail, b.lo, b.hi, d->ptr, d->lo, d->hi, b, c->bufs[in.c].elem, J))
+                if (!make_copy_jobs(it->second.mail, b.lo, b.hi, d->ptr, d->lo, d->hi, b, c->bufs[in.c].elem,
+                                    [&](const CopyJob& J) {
+                                      if (g) g->add_copy(F, J);
+                                      else add_copy(p, Lr + 1, J);
+                                    }))
                   return fail_ctx(c, IGS_ERR_STATE, "bad receive box");
-                if (g) {
-                  g->add_copy(F, J);
-                  g->frees.push_back(it->second.mail);
-                } else {
-                  add_copy(p, Lr + 1, J);
-                  p.at(Lr + 1).frees.push_back(it->second.mail);
-                }
+                if (g) g->frees.push_back(it->second.mail);
+                else p.at(Lr + 1).frees.push_back(it->second.mail);
               }
               c->sends.erase(range.first, range.second);
               h.level[i] = Lr + 1;
@@ -2108,13 +2110,13 @@ extern "C" int igs_read_buffer(igs_ctx* c, uint32_t b, const uint32_t lo[3], con
     if (r) return r;
   }
   Pending p;
+  auto add = [&](const CopyJob& J) { add_copy(p, 1, J); };
   for (const HEntry& e : own) {
     igs_box piece;
     if (!isect(e.lo, e.hi, rl, rh, piece)) continue;
     if (e.v[0] == HOST) {
-      CopyJob J{};
       uint32_t blo[3] = {0, 0, 0}, bhi[3] = {bf.extent[0], bf.extent[1], bf.extent[2]};
-      if (make_copy_job(c->init_dev[b], blo, bhi, stage, rl, rh, piece, bf.elem, J)) add_copy(p, 1, J);
+      make_copy_jobs(c->init_dev[b], blo, bhi, stage, rl, rh, piece, bf.elem, add);
       continue;
     }
     if (e.v[0] >= c->N) continue;  // never written
@@ -2133,8 +2135,7 @@ extern "C" int igs_read_buffer(igs_ctx* c, uint32_t b, const uint32_t lo[3], con
         if (!A.live || A.buffer != b || A.mem != pmem) continue;
         igs_box z;
         if (!isect(A.lo, A.hi, q.lo, q.hi, z)) continue;
-        CopyJob J{};
-        if (make_copy_job(A.ptr, A.lo, A.hi, stage, rl, rh, z, bf.elem, J)) add_copy(p, 1, J);
+        make_copy_jobs(A.ptr, A.lo, A.hi, stage, rl, rh, z, bf.elem, add);
       }
     }
   }
@@ -2153,16 +2154,13 @@ extern "C" int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream) 
   std::vector<CopyJob> v;
   for (uint32_t i = 0; i < n; ++i) {
     const igs_copy_job& j = jobs[i];
-    CopyJob J{};
     for (int d = 0; d < 3; ++d)
       if (j.box.lo[d] < j.src_box.lo[d] || j.box.hi[d] > j.src_box.hi[d] || j.box.lo[d] < j.dst_box.lo[d] ||
           j.box.hi[d] > j.dst_box.hi[d])
         return IGS_ERR_INVALID_ARG;
     if (j.elem_size == 0) continue;  // no bytes (and no rows to split them into)
-    if (!make_copy_job(static_cast<const uint8_t*>(j.src), j.src_box.lo, j.src_box.hi, static_cast<uint8_t*>(j.dst),
-                       j.dst_box.lo, j.dst_box.hi, j.box, j.elem_size, J))
-      continue;
-    v.push_back(J);
+    make_copy_jobs(static_cast<const uint8_t*>(j.src), j.src_box.lo, j.src_box.hi, static_cast<uint8_t*>(j.dst),
+                   j.dst_box.lo, j.dst_box.hi, j.box, j.elem_size, [&](const CopyJob& J) { v.push_back(J); });
   }
   if (v.empty()) return IGS_OK;
   const uint64_t units = place_copies(v.data(), v.size());
