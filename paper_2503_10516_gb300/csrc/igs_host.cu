@@ -1591,6 +1591,7 @@ bool stencil_ok(const igs_ctx* c, const KernelJob& J) {
   if (J.kernel == K_WAVE && (!box_in(J.acc[0].lo, J.acc[0].hi, lo, hi) || !box_in(J.acc[0].plo, J.acc[0].phi, lo, hi)))
     return false;
   for (int d = 0; d < 2; ++d) {
+    if (hi[d] > U.ext[d]) return false;  // items outside the buffer they read
     lo[d] = lo[d] > 0 ? lo[d] - 1 : 0;
     hi[d] = std::min(hi[d] + 1, U.ext[d]);
   }
