@@ -89,13 +89,15 @@ uint32_t igs_nbody_lanes(uint64_t bodies);
 // for jobs that run in one launch.
 uint32_t igs_stencil_tiles(const igs::KernelJob& J, uint32_t rows);
 uint32_t igs_stencil_rows(const igs::KernelJob* jobs, size_t n);
-// 5-point stencil jobs (Jacobi / wave), pre-validated by the host, of at most
-// max_tiles block tiles each; n_jobs <= 65535.
-int igs_launch_stencil(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint32_t max_tiles, void* stream);
+// Sets the rows and first block tile (item_begin) of the jobs of one launch;
+// returns their tiles; *each: the tiles of every job where all have as many, else 0.
+uint32_t igs_stencil_place(igs::KernelJob* jobs, size_t n, uint32_t* each);
+// 5-point stencil jobs (Jacobi / wave), pre-validated by the host and placed by
+// igs_stencil_place.
+int igs_launch_stencil(const igs::KernelJob* jobs_dev, uint32_t n_jobs, uint32_t tiles, uint32_t each, void* stream);
 // One level's stencil jobs and box-copy units in one launch (they are
-// independent by construction of the levels). -1 when the grid would exceed
-// 65535 rows (the caller then launches them separately).
-int igs_launch_level(const igs::KernelJob* sjobs_dev, uint32_t n_sjobs, uint32_t max_tiles,
+// independent by construction of the levels).
+int igs_launch_level(const igs::KernelJob* sjobs_dev, uint32_t n_sjobs, uint32_t tiles, uint32_t each,
                      const igs::CopyJob* cjobs_dev, uint32_t n_cjobs, uint64_t n_units, void* stream);
 // Execution error flags (0 = none; bit 0: a workload kernel met an index
 // outside its allocation, bit 1: a dataflow launch gave up waiting);

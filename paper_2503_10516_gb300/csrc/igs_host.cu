@@ -1014,7 +1014,7 @@ struct LevelWork {
   std::vector<KernelJob> kernels, stencils, nbodies;
   std::vector<void*> frees;
   uint64_t copy_units = 0, kernel_items = 0, bodies = 0, bodies_max = 0;
-  uint32_t stencil_tiles = 0;  // block tiles of the largest stencil job
+  uint32_t stencil_tiles = 0, stencil_each = 0;  // block tiles of the stencil jobs (igs_stencil_place)
 };
 
 // The dataflow graph of one execute call: a node per walked instruction, its
@@ -1253,13 +1253,7 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
     std::copy(w.kernels.begin(), w.kernels.end(), c->h_kjobs[k] + nk);
     nk += w.kernels.size();
     so[L] = nk;
-    if (!w.stencils.empty()) {
-      const uint32_t rows = igs_stencil_rows(w.stencils.data(), w.stencils.size());
-      for (KernelJob& J : w.stencils) {
-        J.lanes = rows;
-        w.stencil_tiles = std::max(w.stencil_tiles, igs_stencil_tiles(J, rows));
-      }
-    }
+    w.stencil_tiles = igs_stencil_place(w.stencils.data(), w.stencils.size(), &w.stencil_each);
     std::copy(w.stencils.begin(), w.stencils.end(), c->h_kjobs[k] + nk);
     nk += w.stencils.size();
     bo[L] = nk;
@@ -1282,10 +1276,10 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
     // a level with both copies and stencil jobs runs as one launch (its
     // instructions are independent of one another); its time counts as
     // workload time and its copy bytes are not in copy_bytes
-    if (!w.copies.empty() && !w.stencils.empty() && w.stencils.size() + 2048 <= 65535) {
+    if (!w.copies.empty() && !w.stencils.empty()) {
       const size_t ev = c->timing ? ev_begin(c, s) : 0;
-      if (igs_launch_level(c->d_kjobs[k] + so[L], (uint32_t)w.stencils.size(), w.stencil_tiles, c->d_cjobs[k] + co[L],
-                           (uint32_t)w.copies.size(), w.copy_units, s))
+      if (igs_launch_level(c->d_kjobs[k] + so[L], (uint32_t)w.stencils.size(), w.stencil_tiles, w.stencil_each,
+                           c->d_cjobs[k] + co[L], (uint32_t)w.copies.size(), w.copy_units, s))
         return fail_ctx(c, IGS_ERR_CUDA, "level launch");
       if (c->timing) ev_end(c, 2, ev, s);
       c->n_launch[2]++;
@@ -1298,10 +1292,9 @@ int run_pending(igs_ctx* c, Pending& p, cudaStream_t s, bool wait) {
         c->n_launch[1]++;
         for (const CopyJob& j : w.copies) c->copy_bytes += 2.0 * j.extent[0] * j.extent[1] * j.extent[2];
       }
-      for (size_t first = 0; first < w.stencils.size(); first += 65535) {
-        const uint32_t n = (uint32_t)std::min<size_t>(65535, w.stencils.size() - first);
+      if (!w.stencils.empty()) {
         const size_t ev = c->timing ? ev_begin(c, s) : 0;
-        if (igs_launch_stencil(c->d_kjobs[k] + so[L] + first, n, w.stencil_tiles, s))
+        if (igs_launch_stencil(c->d_kjobs[k] + so[L], (uint32_t)w.stencils.size(), w.stencil_tiles, w.stencil_each, s))
           return fail_ctx(c, IGS_ERR_CUDA, "stencil launch");
         if (c->timing) ev_end(c, 2, ev, s);
         c->n_launch[2]++;
