@@ -338,9 +338,8 @@ int download_nodes(igs_ctx* c) {
   return IGS_OK;
 }
 
-int check_status(igs_ctx* c) {
-  int r = download_nodes(c);
-  if (r) return r;
+// The status of the nodes as last downloaded.
+int nodes_status(igs_ctx* c) {
   for (uint32_t n = 0; n < c->N; ++n) {
     const NodeDev& nd = c->nodes_host[n];
     if (nd.status == ST_CAPACITY) {
@@ -360,6 +359,36 @@ int check_status(igs_ctx* c) {
   }
   if (c->nodes_host[0].n_rej) return fail_ctx(c, IGS_ERR_OVERLAPPING_WRITE, "a task with overlapping writes was rejected");
   return IGS_OK;
+}
+
+int check_status(igs_ctx* c) {
+  const int r = download_nodes(c);
+  return r ? r : nodes_status(c);
+}
+
+// What lowering changes of node nd (as downloaded; its record at d_node),
+// besides appending to its graph: copies of it to `to`, which advances.
+void save_node(const NodeDev& nd, NodeDev* d_node, size_t& to, std::vector<CopyJob>& jobs) {
+  auto part = [&](const void* p, size_t bytes) {
+    for (size_t at = 0; at < bytes; at += 1u << 30) {
+      CopyJob J{};
+      J.src = static_cast<const uint8_t*>(p) + at;
+      J.dst = reinterpret_cast<uint8_t*>(to + at);  // an offset until there is memory for it
+      J.extent[0] = J.extent[1] = 1;
+      J.extent[2] = (uint32_t)std::min<size_t>(bytes - at, 1u << 30);
+      jobs.push_back(J);
+    }
+    to += (bytes + 255) & ~(size_t)255;
+  };
+  part(d_node, sizeof nd);
+  part(nd.heap, sizeof(uint32_t) * F_COUNT * (size_t)nd.heap_top);
+  part(nd.own_d, sizeof(uint32_t) * kDesc * (2 * nd.cap_buffers + 2 * nd.cap_slots));
+  part(nd.free_slots, sizeof(uint32_t) * nd.cap_slots);
+  part(nd.live, sizeof(uint32_t) * nd.n_live);
+  part(nd.qr_base, sizeof(uint32_t) * F_COUNT * (size_t)nd.qr_n);
+  part(nd.allocs, sizeof(AllocRec) * (size_t)nd.n_alloc);
+  part(nd.queue, nd.q_count ? sizeof(uint32_t) * nd.cap_queue : 0);
+  part(nd.has_succ, nd.n_instr);
 }
 
 int push_item(igs_ctx* c, uint32_t kind, uint32_t arg, uint32_t task) {
@@ -844,10 +873,12 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
   std::vector<Unit> units;
   std::vector<double> work;  // estimated work per unit: pending items plus chunk-accessor pairs per node
   std::vector<std::pair<double, uint32_t>> heavy;  // (work, context) of contexts with several devices
+  std::vector<uint8_t> fresh(n);                   // nothing was lowered yet
   for (uint32_t i = 0; i < n; ++i)
     if (!ctxs[i] || ctxs[i]->server) return fail_ctx(ctxs[i], IGS_ERR_STATE, "a served context cannot be batch-lowered");
   for (uint32_t i = 0; i < n; ++i) {
     igs_ctx* x = ctxs[i];
+    fresh[i] = x->items_up == 0;
     int r = upload_prog(x);
     if (r) return r;
     if (cudaStreamSynchronize(x->stream) != cudaSuccess) return IGS_ERR_CUDA;
@@ -893,8 +924,23 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
   // ten one-warp blocks share: it is the better form while twice the SMs'
   // pace gets through all units well before one warp gets through the longest
   // (24 uneven programs of 142 nodes: 259 ms with one warp per node, 91 ms).
-  uint32_t* pool = nullptr;
+  // Its warps take slabs of a node's heap in another order than one warp (the
+  // front warp ahead of frees), so they may run out of a heap that suffices for
+  // one warp: what the launch changes is saved, and units that fail are lowered
+  // again, from where they were, by one warp.
+  struct Lent {
+    uint32_t* p = nullptr;
+    cudaStream_t s = nullptr;
+    ~Lent() {
+      if (p) cudaFreeAsync(p, s);
+    }
+  } lent;
+  uint32_t*& pool = lent.p;
+  lent.s = c->stream;
   uint32_t pool_blocks = 0, pool_cap = 32, front_cap = 0;
+  std::vector<CopyJob> saves;       // of all units, one after the other
+  std::vector<uint32_t> first_save(1, 0);
+  CopyJob* d_saves = nullptr;
   if (!shape) {
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->cfg.device);
@@ -910,11 +956,31 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
         pool_cap = std::max(pool_cap, ctxs[i]->nodes_host[0].cap_scratch);
         front_cap = std::max(front_cap, ctxs[i]->nodes_host[0].cap_qr);
       }
-      const size_t bytes = sizeof(uint32_t) * igs_lower_pool_words(pool_cap, front_cap) * pool_blocks;
+      const size_t words = sizeof(uint32_t) * igs_lower_pool_words(pool_cap, front_cap) * pool_blocks;
+      size_t bytes = (words + 255) & ~(size_t)255;
+      for (uint32_t i = 0; i < n; ++i) {
+        igs_ctx* x = ctxs[i];
+        int r;
+        if (!fresh[i] && (r = download_nodes(x))) return r;
+        for (uint32_t k = 0; k < x->N; ++k) {
+          save_node(x->nodes_host[k], x->d_nodes + k, bytes, saves);
+          first_save.push_back((uint32_t)saves.size());
+        }
+      }
+      const size_t o_saves = bytes;
+      bytes += sizeof(CopyJob) * saves.size();
       // at most 16 GiB, given back after the launch; without it, one warp per unit
       if (bytes > (size_t)16 << 30 || cudaMallocAsync((void**)&pool, bytes, c->stream) != cudaSuccess) {
         cudaGetLastError();
         pool = nullptr;
+      } else {
+        uint8_t* const base = reinterpret_cast<uint8_t*>(pool);
+        for (CopyJob& J : saves) J.dst = base + reinterpret_cast<size_t>(J.dst);
+        d_saves = reinterpret_cast<CopyJob*>(base + o_saves);
+        const uint64_t copy_units = place_copies(saves.data(), saves.size());
+        CK(cudaMemcpyAsync(d_saves, saves.data(), sizeof(CopyJob) * saves.size(), cudaMemcpyHostToDevice, c->stream));
+        if (igs_launch_copies(d_saves, (uint32_t)saves.size(), copy_units, c->stream))
+          return fail_ctx(c, IGS_ERR_CUDA, "batch launch");
       }
     }
   }
@@ -927,10 +993,8 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
     order[nu] = 0;
     CK(cudaMemcpyAsync(d_order, order.data(), sizeof(uint32_t) * (nu + 1), cudaMemcpyHostToDevice, c->stream));
     if (pool) {
-      const int bad = igs_launch_lower_pool(d_units, nu, d_order, d_order + nu, pool_blocks, pool, pool_cap, front_cap,
-                                            c->stream);
-      cudaFreeAsync(pool, c->stream);
-      if (bad) return fail_ctx(c, IGS_ERR_CUDA, "batch launch");
+      if (igs_launch_lower_pool(d_units, nu, d_order, d_order + nu, pool_blocks, pool, pool_cap, front_cap, c->stream))
+        return fail_ctx(c, IGS_ERR_CUDA, "batch launch");
     } else if (const uint32_t blocks = std::min(shape->persistent_blocks, nu);
                igs_launch_lower_queue(d_units, nu, d_order, d_order + nu, blocks, warps, c->stream))
       return fail_ctx(c, IGS_ERR_CUDA, "batch launch");
@@ -938,9 +1002,40 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
     return fail_ctx(c, IGS_ERR_CUDA, "batch launch");
   }
   CK(cudaStreamSynchronize(c->stream));
+  if (pool) {
+    std::vector<Unit> again;
+    std::vector<CopyJob> back;
+    for (uint32_t i = 0, u = 0; i < n; ++i) {
+      int r = download_nodes(ctxs[i]);
+      if (r) return r;
+      for (uint32_t k = 0; k < ctxs[i]->N; ++k, ++u) {
+        if (ctxs[i]->nodes_host[k].status == ST_OK) continue;
+        again.push_back(units[u]);
+        for (uint32_t s = first_save[u]; s < first_save[u + 1]; ++s) {
+          CopyJob J = saves[s];
+          J.src = saves[s].dst;
+          J.dst = const_cast<uint8_t*>(saves[s].src);
+          back.push_back(J);
+        }
+      }
+    }
+    if (!again.empty()) {
+      const uint64_t copy_units = place_copies(back.data(), back.size());
+      CK(cudaMemcpyAsync(d_saves, back.data(), sizeof(CopyJob) * back.size(), cudaMemcpyHostToDevice, c->stream));
+      CK(cudaMemcpyAsync(d_units, again.data(), sizeof(Unit) * again.size(), cudaMemcpyHostToDevice, c->stream));
+      if (igs_launch_copies(d_saves, (uint32_t)back.size(), copy_units, c->stream) ||
+          igs_launch_lower(d_units, (uint32_t)again.size(), IGS_NONE, c->stream))
+        return fail_ctx(c, IGS_ERR_CUDA, "batch launch");
+      CK(cudaStreamSynchronize(c->stream));
+      for (uint32_t i = 0; i < n; ++i) {
+        int r = download_nodes(ctxs[i]);
+        if (r) return r;
+      }
+    }
+  }
   for (uint32_t i = 0; i < n; ++i) {
     ctxs[i]->launches++;
-    int r = check_status(ctxs[i]);
+    int r = pool ? nodes_status(ctxs[i]) : check_status(ctxs[i]);
     if (r && r != IGS_ERR_OVERLAPPING_WRITE) return fail_ctx(c, r, "context " + std::to_string(i) + ": " + ctxs[i]->err);
   }
   return IGS_OK;

@@ -70,3 +70,51 @@ def test_state_table_runs_out_beside_an_overflowing_plan():
             done.append(heap)
             assert_same_graph(got[0], ref[0], f"heap of {heap} entries")
     assert done and done[0] > 2048  # the range reaches from too small to enough
+
+
+def _rotating_program(nodes, devices, steps):
+    """A new buffer per task, read transposed by the next task and then
+    destroyed: ownership and state tables come and go."""
+    ext = (16, 16, 1)
+    ops = []
+    for k in range(steps):
+        ops.append(("buffer", W.Buffer(2, ext, 4, None, "u32")))
+        accs = [W.Accessor(k, W.WRITE, W.one_to_one())]
+        if k:
+            accs.append(W.Accessor(k - 1, W.READ, W.transposed()))
+        ops.append(("task", W.Task(2, ext, 16, W.K_NOP, accs)))
+        if k > 1:
+            ops.append(("destroy", k - 2))
+    return W.Program(f"rotate{nodes}x{devices}", nodes, devices, 4, 0, ops + [("flush",)])
+
+
+ALONE = (0, 0)  # igs_lower_batch_shaped: one warp per node
+
+
+@pytest.mark.parametrize("parts", [1, 2])
+@pytest.mark.parametrize("nodes,devices", [(1, 4), (4, 1), (4, 2)])
+def test_heap_that_suffices_for_one_warp(nodes, devices, parts):
+    """Helper and front warps take slabs in another order than one warp: where
+    that exhausts a heap that one warp gets by with, in a context's first launch
+    or in a later one, the graph is the oracle's all the same."""
+    prog = _rotating_program(nodes, devices, 12)
+    ref, _ = oracle_graphs(prog)
+    cut = len(prog.ops) // 2
+    pieces = [prog.ops[:cut], prog.ops[cut:]] if parts == 2 else [prog.ops]
+
+    def lower(heap, shape):
+        return _lower(prog, pieces, shape, map_heap=heap, scratch_capacity=1024)
+    too_small, least = 128, 8192
+    assert lower(too_small, ALONE) is None and lower(least, ALONE) is not None
+    while least - too_small > 32:
+        mid = (too_small + least) // 64 * 32
+        if lower(mid, ALONE) is None:
+            too_small = mid
+        else:
+            least = mid
+    assert lower(too_small, None) is None
+    for heap in range(least, least + 512, 32):
+        got = lower(heap, None)
+        assert got is not None, f"a heap of {least} entries suffices for one warp, {heap} do not"
+        for n in range(nodes):
+            assert_same_graph(got[n], ref[n], f"node {n}, heap of {heap} entries")
