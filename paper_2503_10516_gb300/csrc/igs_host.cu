@@ -15,6 +15,7 @@
 #include <thread>
 #include <cstring>
 #include <deque>
+#include <functional>
 #include <map>
 #include <unordered_map>
 #include <string>
@@ -874,6 +875,12 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
   std::vector<double> work;  // estimated work per unit: pending items plus chunk-accessor pairs per node
   std::vector<std::pair<double, uint32_t>> heavy;  // (work, context) of contexts with several devices
   std::vector<uint8_t> fresh(n);                   // nothing was lowered yet
+  // one warp's time for a context's pending work on a node, in us: for a
+  // submission, a task's exchange with each node, a chunk-accessor pair (waves,
+  // N-body steps: within a third), where transposed accesses fragment the maps
+  // (uneven batches of 255 and 497 nodes: within a tenth)
+  constexpr double kItemUs = 10, kTaskNodeUs = 30, kPairUs = 5.8, kFragmentedPairUs = 23;
+  std::vector<double> alone_us(n);
   for (uint32_t i = 0; i < n; ++i)
     if (!ctxs[i] || ctxs[i]->server) return fail_ctx(ctxs[i], IGS_ERR_STATE, "a served context cannot be batch-lowered");
   for (uint32_t i = 0; i < n; ++i) {
@@ -882,15 +889,23 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
     int r = upload_prog(x);
     if (r) return r;
     if (cudaStreamSynchronize(x->stream) != cudaSuccess) return IGS_ERR_CUDA;
-    double w = 0;
+    double w = 0, items = 0, tasks = 0;
+    bool fragmented = false;
     for (size_t k = x->nodes_host[0].cursor; k < x->items.size(); ++k) {
       w += 1;
+      items += 1;
       if (x->items[k].kind == IT_TASK) {
+        tasks += 1;
         const igs_task& t = x->tasks[x->items[k].task];
         const double chunks = (double)(t.num_chunks & 0xFFFFu) * std::max(1u, t.num_chunks >> 16);
         w += chunks * t.num_accessors / x->N;
+        for (uint32_t a = 0; a < t.num_accessors; ++a)
+          for (int d = 1; d < 3; ++d)
+            if (t.acc[a].dim[d].kind == IGS_MAP_AFFINE && t.acc[a].dim[d].a == 0) fragmented = true;
       }
     }
+    alone_us[i] = items * kItemUs + (x->N > 1 ? tasks * x->N * kTaskNodeUs : 0) +
+                  (w - items) * (fragmented && x->N * x->D > 1 ? kFragmentedPairUs : kPairUs);
     for (uint32_t k = 0; k < x->N; ++k) {
       units.push_back(Unit{x->d_nodes + k, x->d_prog});
       work.push_back(w);
@@ -919,11 +934,17 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
   }
   CK(cudaMemcpyAsync(d_units, units.data(), sizeof(Unit) * units.size(), cudaMemcpyHostToDevice, c->stream));
   const uint32_t nu = (uint32_t)units.size();
-  // A launch ends with its longest unit. A block of helper and front warps
-  // lowers a unit about twice as fast as one warp, but takes an SM that about
-  // ten one-warp blocks share: it is the better form while twice the SMs'
-  // pace gets through all units well before one warp gets through the longest
-  // (24 uneven programs of 142 nodes: 259 ms with one warp per node, 91 ms).
+  // A launch ends with its longest unit, and a block of helper and front warps
+  // lowers a unit two to three times as fast as one warp (waves, N-body steps,
+  // batches of 50 to 500 units; growing rows a tenth), but needs scratch, which
+  // the driver maps and unmaps for every launch: 0.11 ms and 2.1 us a MiB. It is
+  // the better form where what it takes off the longest unit, by one warp's
+  // estimated time, exceeds that. Many equal units end as soon either way (about
+  // 25 wave programs a ms).
+  // igs_lower_batch, one warp / lent warps: one 1 x 4 context, 4 wave tasks 1.11
+  // / 0.55 ms; 24 uneven programs (255 nodes) 133 / 72 ms, 60 (497 nodes) 89 / 59;
+  // but one 1 x 1 context, one task 0.11 / 0.27 ms; eight 4 x 4 contexts, one task
+  // 0.64 / 2.8 ms; 40 of 4 x 1, 16 tasks (160 nodes) 4.6 / 8.5 ms.
   // Its warps take slabs of a node's heap in another order than one warp (the
   // front warp ahead of frees), so they may run out of a heap that suffices for
   // one warp: what the launch changes is saved, and units that fail are lowered
@@ -932,7 +953,9 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
     uint32_t* p = nullptr;
     cudaStream_t s = nullptr;
     ~Lent() {
-      if (p) cudaFreeAsync(p, s);
+      if (!p) return;
+      cudaFreeAsync(p, s);
+      cudaStreamSynchronize(s);  // back to the driver before the call returns
     }
   } lent;
   uint32_t*& pool = lent.p;
@@ -944,19 +967,24 @@ int igs_lower_batch_shaped(igs_ctx* const* ctxs, uint32_t n, const igs_batch_sha
   if (!shape) {
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->cfg.device);
+    std::vector<double> helped;  // of every unit
     double sum = 0, longest = 0;
-    for (double w : work) {
-      sum += w;
-      longest = std::max(longest, w);
+    for (uint32_t i = 0; i < n; ++i) {
+      const double us = alone_us[i] / (ctxs[i]->D > 2 ? 3.0 : 2.0);
+      helped.insert(helped.end(), ctxs[i]->N, us);
+      longest = std::max(longest, alone_us[i]);
+      sum += us * ctxs[i]->N;
     }
-    const double helped = std::max(longest / 2, sum / (2.0 * sms)), alone = std::max(longest, sum / (10.0 * sms));
-    if (helped < 0.8 * alone) {
-      pool_blocks = std::min<uint32_t>(nu, (uint32_t)sms);
-      for (uint32_t i = 0; i < n; ++i) {
-        pool_cap = std::max(pool_cap, ctxs[i]->nodes_host[0].cap_scratch);
-        front_cap = std::max(front_cap, ctxs[i]->nodes_host[0].cap_qr);
-      }
-      const size_t words = sizeof(uint32_t) * igs_lower_pool_words(pool_cap, front_cap) * pool_blocks;
+    std::sort(helped.begin(), helped.end(), std::greater<double>());
+    double with = std::max(helped[0], 1.1 * sum / sms);  // busy SMs slow one another
+    if (nu > (uint32_t)sms) with = std::max(with, helped[sms - 1] + helped[sms]);  // two in one block
+    pool_blocks = std::min<uint32_t>(nu, (uint32_t)sms);
+    for (uint32_t i = 0; i < n; ++i) {
+      pool_cap = std::max(pool_cap, ctxs[i]->nodes_host[0].cap_scratch);
+      front_cap = std::max(front_cap, ctxs[i]->nodes_host[0].cap_qr);
+    }
+    const size_t words = sizeof(uint32_t) * igs_lower_pool_words(pool_cap, front_cap) * pool_blocks;
+    if (longest - with > 1.25 * (110.0 + 2.1 * (double)(words >> 20))) {  // the cost, with a margin
       size_t bytes = (words + 255) & ~(size_t)255;
       for (uint32_t i = 0; i < n; ++i) {
         igs_ctx* x = ctxs[i];

@@ -118,3 +118,32 @@ def test_heap_that_suffices_for_one_warp(nodes, devices, parts):
         assert got is not None, f"a heap of {least} entries suffices for one warp, {heap} do not"
         for n in range(nodes):
             assert_same_graph(got[n], ref[n], f"node {n}, heap of {heap} entries")
+
+
+@pytest.mark.parametrize("nodes,devices,chunks,tasks,lent", [
+    (1, 1, 2, 1, False), (1, 1, 2, 4, False), (4, 2, 16, 1, False), (1, 2, 96, 1, True), (1, 2, 96, 2, True),
+    (1, 1, 96, 3, True), (4, 2, 16, 24, True), (1, 4, 16, 9, True)])
+def test_form_of_a_batch(nodes, devices, chunks, tasks, lent):
+    """Warps are lent where there is enough to lower, also for one, two and
+    three items; small calls keep one warp per node. Lowered twice, so that the
+    second call is not the context's first."""
+    from paper_2503_10516_gb300 import igs
+    ext = (max(chunks, 8), 8, 1)
+    ops = [("buffer", W.Buffer(2, ext, 4, None, "u32")) for _ in range(2)]
+    for k in range(tasks):
+        accs = [W.Accessor(k % 2, W.WRITE, W.one_to_one())]
+        if k:
+            accs.append(W.Accessor((k + 1) % 2, W.READ, W.neighborhood(1)))
+        ops.append(("task", W.Task(2, ext, chunks, W.K_NOP, accs)))
+    prog = W.Program("form", nodes, devices, 4, 0, ops + ops[2:])
+    ref, _ = oracle_graphs(prog)
+    c = igs.Context(nodes, devices, 4, 0, mode=igs.MODE_BATCHED)
+    phases = [0]
+    for part in (ops, ops[2:]):
+        _submit(c, part)
+        igs.lower_batch([c])
+        phases.append(c.profile()["n_shared_phases"])
+        assert (phases[-1] > phases[-2]) == lent
+    for n in range(nodes):
+        assert_same_graph(c.graph(n), ref[n], f"node {n}")
+    c.close()
