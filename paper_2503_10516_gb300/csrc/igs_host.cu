@@ -2269,6 +2269,7 @@ extern "C" int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream) 
   igs_ctx* c = nullptr;
   if (!jobs && n) return IGS_ERR_INVALID_ARG;
   std::vector<CopyJob> v;
+  v.reserve(n);
   for (uint32_t i = 0; i < n; ++i) {
     const igs_copy_job& j = jobs[i];
     for (int d = 0; d < 3; ++d)

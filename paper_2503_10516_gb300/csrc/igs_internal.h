@@ -170,9 +170,11 @@ constexpr uint32_t kCopyWarps = 8;  // warps of a copying block
 // Jobs that travel in the kernel's parameters (4 KB).
 constexpr uint32_t kCopyFewJobs = 44;
 
+// (Most jobs are one unit, and a division takes the host longer than the rest.)
 inline uint64_t copy_units(const CopyJob& j) {
-  return (uint64_t)j.extent[0] * ((j.extent[1] - 1) / j.rows_unit + 1) *
-         ((j.extent[2] + j.seg_bytes - 1) / j.seg_bytes);
+  const uint32_t groups = j.extent[1] <= j.rows_unit ? 1u : (j.extent[1] - 1) / j.rows_unit + 1;
+  const uint32_t segs = j.extent[2] <= j.seg_bytes ? 1u : (j.extent[2] + j.seg_bytes - 1) / j.seg_bytes;
+  return (uint64_t)j.extent[0] * groups * segs;
 }
 
 // Splits a job into work units of about `unit` bytes (a power of two).
@@ -196,7 +198,7 @@ inline void split_copy(CopyJob& j, uint32_t unit) {
     j.dst_stride[1] = t;
   }
   j.rows_unit = 1;
-  if (run < kCopyShortRow) j.rows_unit = (uint32_t)(unit / run);  // at most 2^16 elements
+  if (run < kCopyShortRow) j.rows_unit = j.extent[1] == 1 ? 1u : unit / j.extent[2];  // at most 2^16 elements
   else if (kCopyWarps * run <= 4 * unit) j.rows_unit = kCopyWarps;  // else the warps share a piece of one row
   j.seg_bytes = unit;
 }

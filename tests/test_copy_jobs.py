@@ -69,3 +69,24 @@ def test_buffer_longer_than_a_job(executor):
         got = c.read_buffer(b, (0, 0, 0), ext, 4).view(np.float32).reshape(-1)
         assert np.array_equal(got, data), b
     c.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_jobs", [45, 46, 300])
+@pytest.mark.parametrize("order", ["ascending", "descending", "mixed"])
+def test_jobs_of_unequal_size(order, n_jobs):
+    """Many jobs of 4 bytes to 300 KB (one unit to dozens) in one launch: a
+    block finds its job where even sizes would put it, or by search."""
+    import torch
+    from paper_2503_10516_gb300 import igs
+    rng = np.random.default_rng(n_jobs)
+    sizes = np.sort(np.exp(rng.uniform(0, np.log(75000), n_jobs)).astype(np.int64))
+    if order != "ascending":
+        sizes = sizes[::-1] if order == "descending" else rng.permutation(sizes)
+    at = np.concatenate([[0], np.cumsum(sizes)])
+    src = torch.arange(int(at[-1]), dtype=torch.int32, device="cuda")
+    dst = torch.full((int(at[-1]) + 1,), -1, dtype=torch.int32, device="cuda")
+    box = [(0, 0, 0, 1, 1, int(s)) for s in sizes]
+    igs.box_copy([(src.data_ptr() + 4 * int(a), b, dst.data_ptr() + 4 * int(a) + 4, b, b, 4) for a, b in zip(at, box)],
+                 torch.cuda.current_stream().cuda_stream)
+    assert torch.equal(dst[1:], src) and int(dst[0]) == -1
