@@ -318,6 +318,12 @@ int igs_bounds_errors(igs_ctx* ctx, igs_bounds_error* out, uint32_t cap, uint32_
  * giving up (a defect), IGS_ERR_INVALID_ARG / IGS_ERR_CUDA otherwise. */
 int igs_selftest_flow_wait(uint32_t wait_ms);
 
+/* Self-test of the N-body step's arithmetic on the current device: *differing
+ * becomes the number of floats in [2^-20, 2^80), the range in which the step
+ * evaluates 1 / (x * sqrt(x)) by its own sequence of operations, for which that
+ * differs in any bit from the rounded square root, product and quotient. */
+int igs_selftest_nbody_weight(uint64_t* differing);
+
 /* Lowers every pending submission and executes the whole graph with the
  * scheduler running ahead of the executor (Sec. 4: instruction generation
  * runs concurrently with execution, off the critical path): one launch on the

@@ -103,3 +103,5 @@ int igs_launch_level(const igs::KernelJob* sjobs_dev, uint32_t n_sjobs, uint32_t
 // outside its allocation, bit 1: a dataflow launch gave up waiting);
 // optionally clears them.
 int igs_exec_error(bool clear);
+// The floats for which the N-body step's weight differs from the IEEE operations.
+int igs_check_weight(uint64_t* differing);

@@ -658,6 +658,11 @@ int igs_exec_stats(igs_ctx* c, double out[8]) {
   return IGS_OK;
 }
 
+int igs_selftest_nbody_weight(uint64_t* differing) {
+  if (!differing) return IGS_ERR_INVALID_ARG;
+  return igs_check_weight(differing) ? IGS_ERR_CUDA : IGS_OK;
+}
+
 int igs_selftest_flow_wait(uint32_t wait_ms) {
   if (wait_ms < 1 || wait_ms > 10000) return IGS_ERR_INVALID_ARG;
   // layout: control block, two nodes, successor list {1, 0}, pending {1, 1},

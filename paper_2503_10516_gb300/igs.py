@@ -34,7 +34,7 @@ EXPORTS = ("igs_create", "igs_destroy", "igs_create_buffer", "igs_destroy_buffer
            "igs_set_timing", "igs_stats", "igs_profile", "igs_lower_static", "igs_submit_epoch",
            "igs_serve_create", "igs_serve_destroy", "igs_serve_attach", "igs_serve_start", "igs_serve_progress",
            "igs_serve_detach", "igs_serve_stop", "igs_run", "igs_lower_batch_shaped", "igs_set_executor",
-           "igs_exec_stats", "igs_selftest_flow_wait", "igs_bounds_errors", "igs_serve_replay",
+           "igs_exec_stats", "igs_selftest_flow_wait", "igs_selftest_nbody_weight", "igs_bounds_errors", "igs_serve_replay",
            "igs_horizon_plan", "igs_serve_enqueue", "igs_serve_stats", "igs_serve_replay_ex",
            "igs_replay_plain", "igs_set_item_times", "igs_item_times")
 EXEC_LEVELS, EXEC_DATAFLOW = 0, 1  # IGS_EXEC_*
@@ -129,6 +129,7 @@ def lib():
         L.igs_set_executor.argtypes = [vp, u32]
         L.igs_exec_stats.argtypes = [vp, ctypes.POINTER(ctypes.c_double)]
         L.igs_selftest_flow_wait.argtypes = [u32]
+        L.igs_selftest_nbody_weight.argtypes = [ctypes.POINTER(ctypes.c_uint64)]
         L.igs_bounds_errors.argtypes = [vp, vp, u32, P32]
         L.igs_serve_replay.argtypes = [vp, ctypes.POINTER(vp), u32, vp, u32, u32, vp, vp]
         L.igs_serve_replay_ex.argtypes = [vp, ctypes.POINTER(vp), u32, vp, u32, u32, u32, vp, vp]
@@ -512,6 +513,16 @@ def selftest_flow_wait(wait_ms: int) -> int:
     nothing ever becomes ready); returns the status code (IGS_ERR_TIMEOUT
     when the wait gave up as designed)."""
     return lib().igs_selftest_flow_wait(wait_ms)
+
+
+def selftest_nbody_weight() -> int:
+    """Number of floats for which the N-body step's weight differs from the
+    rounded operations (every float it is used for is compared)."""
+    n = ctypes.c_uint64(0)
+    r = lib().igs_selftest_nbody_weight(ctypes.byref(n))
+    if r != IGS_OK:
+        raise IgsError(r, "selftest_nbody_weight")
+    return n.value
 
 
 def lower_batch(ctxs: Sequence[Context], shape: Optional[Tuple[int, ...]] = None):
