@@ -2311,6 +2311,7 @@ extern "C" int igs_serve_create(const igs_serve_config* cfg, igs_server** out) {
   if (!cfg || !out || cfg->max_slots == 0) return IGS_ERR_INVALID_ARG;
   *out = nullptr;
   if (cudaSetDevice(cfg->device) != cudaSuccess) return IGS_ERR_CUDA;
+  igs_exec_preload();
   igs_server* s = new igs_server();
   s->cfg = *cfg;
   if (s->cfg.idle_timeout_ms == 0) s->cfg.idle_timeout_ms = 10000;
@@ -2319,7 +2320,16 @@ extern "C" int igs_serve_create(const igs_serve_config* cfg, igs_server** out) {
       cudaHostAlloc(&s->stop, sizeof(uint32_t), cudaHostAllocMapped) != cudaSuccess ||
       cudaHostGetDevicePointer((void**)&s->d_slots, s->slots, 0) != cudaSuccess ||
       cudaHostGetDevicePointer((void**)&s->d_stop, s->stop, 0) != cudaSuccess ||
-      cudaEventCreateWithFlags(&s->done_ev, cudaEventDisableTiming) != cudaSuccess) {
+      cudaEventCreateWithFlags(&s->done_ev, cudaEventDisableTiming) != cudaSuccess ||
+      // a kernel's first launch loads its module and may enlarge the device's
+      // local memory, which waits for running kernels: every form of lowering
+      // that other contexts may take while the loop runs is launched before it
+      // (each is a module, and a stack frame, of its own)
+      igs_launch_lower(nullptr, 0, IGS_NONE, s->stream, false, nullptr, true) ||
+      igs_launch_lower_alone(nullptr, 0, IGS_NONE, s->stream, nullptr) ||
+      igs_launch_lower_queue(nullptr, 0, nullptr, nullptr, 1, 1, s->stream) ||
+      igs_launch_lower_pool(nullptr, 0, nullptr, nullptr, 1, nullptr, 32, 0, s->stream) ||
+      cudaStreamSynchronize(s->stream) != cudaSuccess) {
     igs_serve_destroy(s);
     return IGS_ERR_CUDA;
   }

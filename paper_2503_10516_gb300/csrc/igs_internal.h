@@ -222,7 +222,8 @@ inline uint64_t place_copies(CopyJob* jobs, size_t n) {
 
 }  // namespace igs
 
-// Device entry points implemented in the .cu translation units.
+// Device entry points implemented in the .cu translation units. A lowering
+// launch of no units is one block that does nothing (igs_serve_create).
 // Persistent blocks of `warps` warps (1..kQueueWarps) pulling units from a
 // device work queue (*head, zero before the launch) in the order order_dev
 // (null = index order); extra warps help nodes that have helper scratch.

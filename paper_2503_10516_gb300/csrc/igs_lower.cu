@@ -4957,6 +4957,7 @@ template <uint32_t kThreads>
 __global__ void __launch_bounds__(kThreads, 1) lower_kernel(const Unit* units, uint32_t n_units, uint32_t max_items,
                                                            volatile uint32_t* progress) {
   __shared__ BlockShared sh;
+  if (blockIdx.x >= n_units) return;
   if (threadIdx.x == 0) {
     sh.lent = 0;
     unit_begin(sh, units[blockIdx.x], blockDim.x >> 5, max_items);
@@ -4976,6 +4977,7 @@ __global__ void __launch_bounds__(kReserveThreads, 1) lower_pool_kernel(const Un
                                                                     uint32_t* scratch, size_t slot_words,
                                                                     uint32_t front_cap) {
   __shared__ BlockShared sh;
+  if (n_units == 0) return;
   uint32_t* const mine = scratch + blockIdx.x * slot_words;
   for (;;) {
     if (threadIdx.x == 0) {
@@ -5009,6 +5011,7 @@ __global__ void __launch_bounds__(kReserveThreads, 1) lower_pool_kernel(const Un
 __global__ void __launch_bounds__(32 * kQueueWarps) lower_queue_kernel(const Unit* units, uint32_t n_units,
                                                                       const uint32_t* order, uint32_t* head) {
   __shared__ BlockShared sh;
+  if (n_units == 0) return;
   const uint32_t warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const uint32_t workers = nw < kMaxWorkers ? nw : kMaxWorkers;
   if (threadIdx.x == 0) {
@@ -5188,13 +5191,12 @@ int igs_launch_serve(igs::ServeSlot* slots, uint32_t n_slots, volatile uint32_t*
 int igs_launch_lower_queue(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                            uint32_t blocks, uint32_t warps, void* stream) {
   if (warps < 1 || warps > igs::kQueueWarps) return -1;
-  if (n_units == 0) return 0;
   static bool carveout = false;
   if (!carveout) {
     cudaFuncSetAttribute(igs::lower_queue_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
     carveout = true;
   }
-  igs::lower_queue_kernel<<<blocks, 32 * warps, 0, (cudaStream_t)stream>>>(units_dev, n_units, order_dev, head_dev);
+  igs::lower_queue_kernel<<<n_units ? blocks : 1, 32 * warps, 0, (cudaStream_t)stream>>>(units_dev, n_units, order_dev, head_dev);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 #endif
@@ -5210,13 +5212,12 @@ size_t igs_lower_pool_words(uint32_t cap_scratch, uint32_t front_cap) {
 int igs_launch_lower_pool(const igs::Unit* units_dev, uint32_t n_units, const uint32_t* order_dev, uint32_t* head_dev,
                           uint32_t blocks, uint32_t* scratch_dev, uint32_t cap_scratch, uint32_t front_cap,
                           void* stream) {
-  if (n_units == 0) return 0;
   static bool carveout = false;
   if (!carveout) {
     cudaFuncSetAttribute(igs::lower_pool_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
     carveout = true;
   }
-  igs::lower_pool_kernel<<<blocks, 32 * (igs::kMaxWorkers + 1), 0, (cudaStream_t)stream>>>(
+  igs::lower_pool_kernel<<<n_units ? blocks : 1, 32 * (igs::kMaxWorkers + 1), 0, (cudaStream_t)stream>>>(
       units_dev, n_units, order_dev, head_dev, scratch_dev, igs_lower_pool_words(cap_scratch, front_cap), front_cap);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -5232,14 +5233,14 @@ int igs_launch_lower_alone(const igs::Unit* units_dev, uint32_t n_units, uint32_
     cudaFuncSetAttribute(igs::lower_kernel<igs::kAloneThreads>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
     carveout = true;
   }
-  igs::lower_kernel<igs::kAloneThreads><<<n_units, 32, 0, (cudaStream_t)stream>>>(units_dev, n_units, max_items, progress);
+  igs::lower_kernel<igs::kAloneThreads><<<n_units ? n_units : 1, 32, 0, (cudaStream_t)stream>>>(units_dev, n_units,
+                                                                                            max_items, progress);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 #endif
 #if IGS_LOWER_IS(0)
 int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_items, void* stream, bool reserve,
                      volatile uint32_t* progress, bool workers) {
-  if (n_units == 0) return 0;
   if (!reserve && !workers) return igs_launch_lower_alone(units_dev, n_units, max_items, stream, progress);
   static bool carveout = false;
   if (!carveout) {
@@ -5248,8 +5249,8 @@ int igs_launch_lower(const igs::Unit* units_dev, uint32_t n_units, uint32_t max_
   }
   // kMaxWorkers warps plus the front warp of pipelined launches
   const uint32_t threads = reserve ? igs::kReserveThreads : 32 * (igs::kMaxWorkers + 1);
-  igs::lower_kernel<igs::kReserveThreads><<<n_units, threads, 0, (cudaStream_t)stream>>>(units_dev, n_units, max_items,
-                                                                                        progress);
+  igs::lower_kernel<igs::kReserveThreads><<<n_units ? n_units : 1, threads, 0, (cudaStream_t)stream>>>(
+      units_dev, n_units, max_items, progress);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 #endif
