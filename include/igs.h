@@ -343,11 +343,17 @@ int igs_run(igs_ctx* ctx, uint32_t window);
 int igs_read_buffer(igs_ctx* ctx, uint32_t buffer, const uint32_t lo[3], const uint32_t hi[3], void* host_dst);
 
 /* Lowers the pending submissions of n contexts in ONE persistent launch (all
- * contexts must share a device). Waits for completion. */
+ * contexts must share a device). Waits for completion.
+ *   Where that ends the launch sooner, blocks of several warps lower the nodes;
+ * their scratch and a copy of the nodes' state (tens of MB for each of at most
+ * as many blocks as the device has SMs, 16 GiB in all) are allocated for the
+ * call. One warp lowers a node where they pay less than they cost or cannot be
+ * had, and again, from its state before the call, each node that fails with
+ * them: what one warp lowers is lowered. */
 int igs_lower_batch(igs_ctx* const* ctxs, uint32_t n);
 
-/* Batched lowering shapes. persistent_blocks = 0: one block per (program,
- * node) unit, as igs_lower_batch (the other fields are ignored). Otherwise
+/* Batched lowering shapes. persistent_blocks = 0: one block of one warp per
+ * (program, node) unit (the other fields are ignored). Otherwise
  * that many persistent blocks of `warps` warps (1..8; 0 counts as 1) take
  * units from a device work queue, in the order `order` gives:
  * IGS_ORDER_SUBMISSION (contexts, then nodes) or IGS_ORDER_LONGEST_FIRST
@@ -528,7 +534,7 @@ int igs_box_copy(const igs_copy_job* jobs, uint32_t n, void* stream);
  * device). igs_lower_static lowers a whole program (buffers, tasks, flushes,
  * buffer destructions, lookahead changes, in `ops` order) on every node into
  * caller-owned DEVICE output arrays, using file-scope device arrays as its
- * only scratch (32 MiB, and 42 MiB for the warps that share a node's lowering
+ * only scratch (32 MiB, and 40.5 MiB for the warps that share a node's lowering
  * in programs of up to 8 nodes): it calls no cudaMalloc, cudaFree or other
  * allocating routine. Every GPU that loads the library holds them until exit.
  *   Limits: at most 16 buffers; per node at most 128 live allocations and a

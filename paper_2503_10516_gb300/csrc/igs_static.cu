@@ -33,12 +33,13 @@ constexpr uint32_t kBuffers = 16, kHeap = 1u << 15, kSlots = 128, kQr = 2048, kS
 constexpr uint32_t kAlloc = 4096, kQueue = 4096, kRej = 256;
 
 // Scratch of the warps that share a node's lowering (helper warps and the
-// front warp of igs_lower.cu), for programs of at most kHelpedNodes nodes: 42
-// MiB. Programs of more nodes already fill as many SMs with one warp each.
+// front warp of igs_lower.cu), for programs of at most kHelpedNodes nodes, which
+// its size sets: 40.5 MiB. Programs of more nodes are lowered by one warp a node.
 constexpr uint32_t kHelpedNodes = 8;
 constexpr size_t kHelperBytes =
     (size_t)igs::kScratchSets * igs::kHelperTables * igs::F_COUNT * kScratch * sizeof(uint32_t);
 __device__ __align__(256) uint8_t g_static_helpers[kHelpedNodes * kHelperBytes];
+static_assert(sizeof g_static_helpers == 81ull << 19, "igs.h states 40.5 MiB");
 
 size_t tbytes(uint32_t cap) { return (size_t)igs::F_COUNT * cap * sizeof(uint32_t); }
 
