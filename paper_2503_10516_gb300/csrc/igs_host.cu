@@ -2186,15 +2186,21 @@ int read_slab(igs_ctx* c, const NodeDev& nd, const uint32_t* desc, std::vector<H
 // Has the system back the pages of the caller's array. A result array is
 // often fresh memory, and a page that nobody has touched costs a fault of the
 // device-to-host copy, which populating them ahead spares (three arrays of 29
-// MB: 50 -> 4.3 ms; three of 67 MB: 11.4 -> 8.9 ms). Best effort: it works
-// without.
+// MB: 50 -> 4.3 ms; three of 67 MB: 11.4 -> 8.9 ms). A large array that is there
+// already, by four of its pages, is left alone: walking all of them took 25 us
+// of 260 for 4 MB, 0.1 ms of 2.0 for 256 MB. Best effort: it works without.
 void populate_pages(void* p, size_t n) {
 #ifndef MADV_POPULATE_WRITE
   constexpr int MADV_POPULATE_WRITE = 23;
 #endif
   const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
   const uintptr_t lo = (uintptr_t)p & ~(page - 1), hi = ((uintptr_t)p + n + page - 1) & ~(page - 1);
-  (void)madvise(reinterpret_cast<void*>(lo), hi - lo, MADV_POPULATE_WRITE);
+  bool there = n >= (1u << 20);
+  for (uintptr_t k = 0, last = (hi - lo) / page - 1; there && k < 4; ++k) {
+    unsigned char in = 1;
+    there = mincore(reinterpret_cast<void*>(lo + last * k / 3 * page), page, &in) || (in & 1);
+  }
+  if (!there) (void)madvise(reinterpret_cast<void*>(lo), hi - lo, MADV_POPULATE_WRITE);
 }
 
 bool isect(const uint32_t alo[3], const uint32_t ahi[3], const uint32_t blo[3], const uint32_t bhi[3], igs_box& o) {
