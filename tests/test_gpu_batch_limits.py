@@ -147,3 +147,26 @@ def test_form_of_a_batch(nodes, devices, chunks, tasks, lent):
     for n in range(nodes):
         assert_same_graph(c.graph(n), ref[n], f"node {n}")
     c.close()
+
+
+@pytest.mark.parametrize("devices", [2, 3])
+def test_coherence_plan_overflows(devices):
+    """Every copy of the fourth task overwrites rows that up to 100 kernels of
+    the second read: some 10^4 edges for the one or two workers that plan a
+    memory, 2048 in a stage. The phase is taken by one warp, then the kernels."""
+    from paper_2503_10516_gb300 import igs
+    ext = (200, 2, 1)
+    ops = [("buffer", W.Buffer(2, ext, 4, None, "u32")) for _ in range(2)]
+    for k in range(4):
+        accs = [W.Accessor(k % 2, W.WRITE, W.one_to_one())]
+        if k:
+            accs.append(W.Accessor((k + 1) % 2, W.READ, W.all_mapper()))
+        ops.append(("task", W.Task(2, ext, 200, W.K_NOP, accs)))
+    prog = W.Program("overwrite", 1, devices, 100, 2, ops + [("flush",)])
+    ref, _ = oracle_graphs(prog)
+    c = igs.Context(1, devices, 100, 2, mode=igs.MODE_BATCHED, scratch_capacity=512)
+    _submit(c, prog.ops)
+    igs.lower_batch([c])
+    assert c.profile()["n_shared_phases"] > 0
+    assert_same_graph(c.graph(0), ref[0])
+    c.close()
